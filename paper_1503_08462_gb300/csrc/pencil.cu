@@ -2466,89 +2466,160 @@ __global__ void __launch_bounds__(kSrqiThreads) k_srqi_check(int m, int q, const
   }
 }
 
-// Fallback: H = [[Theta, Ft L^-T], [L^-1 Ft^T, L^-1 Tt L^-T]] with S = L L^T
-// (float-float Cholesky; status = ENOTSPD when S is not positive definite).
-__global__ void __launch_bounds__(512) k_std_form(int m, int q, const double* __restrict__ thg,
-                                                  const df* __restrict__ Ft, const df* __restrict__ Tt,
-                                                  const df* __restrict__ St, df* __restrict__ L, df* __restrict__ Xs,
-                                                  double* __restrict__ H, int* status, const int* skip,
-                                                  int* nfallback) {
-  if (skip && *skip) return;
-  if (threadIdx.x == 0 && nfallback) atomicAdd(nfallback, 1);
-  extern __shared__ __align__(16) unsigned char fraw[];
-  df* Ls = reinterpret_cast<df*>(fraw);  // q x q
-  __shared__ int bad;
-  const int tid = threadIdx.x, nt = blockDim.x;
-  const int n = m + q;
-  const long long N = n;
-  if (tid == 0) bad = 0;
-  for (int idx = tid; idx < q * q; idx += nt) {
-    const int r = idx / q, c = idx % q;
-    Ls[idx] = c <= r ? St[idx] : df{0.f, 0.f};
-  }
-  __syncthreads();
-  for (int k = 0; k < q; ++k) {
-    if (tid == 0) {
-      const df d = Ls[k * q + k];
-      if (!(d.hi > 0.f)) {
-        bad = 1;
-        Ls[k * q + k] = df{1.f, 0.f};
-      } else {
-        Ls[k * q + k] = df_sqrt(d);
+// Column solves of the standard form: one warp per right-hand side, row i = lane + 32 r in slot r of the
+// lane's registers (q <= 128: four slots).  Each step's solved entry goes to the warp by a shuffle and every
+// remaining row takes its product at once, so a step costs one dependent multiply, shuffle and compensated
+// product (~100 cycles) instead of a dot product per row and a division (multiplication by 1 / l_kk instead).
+constexpr int kStdSlots = kStdMaxQ / 32;
+
+// x = L^-1 acc, forward; L (row stride ld, shared), dinv = 1 / diag(L)
+__device__ __forceinline__ void warp_solve_lower(const df* L, int ld, const df* dinv, int q, df_acc* acc, df* x) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int s = 0; s < kStdSlots; ++s) {
+    if (32 * s >= q) break;
+    const int ke = min(q - 32 * s, 32);
+    for (int t = 0; t < ke; ++t) {
+      const int k = 32 * s + t;
+      const df xk = shfl_df(df_mul(acc[s].value(), dinv[k]), t);
+      if (lane == t) x[s] = xk;
+      const df nx = df_neg(xk);
+#pragma unroll
+      for (int r = s; r < kStdSlots; ++r) {
+        const int i = lane + 32 * r;
+        if (i > k && i < q) acc[r].fma(L[i * ld + k], nx);
       }
     }
-    __syncthreads();
-    const df inv = df_div(df{1.f, 0.f}, Ls[k * q + k]);
-    for (int i = k + 1 + tid; i < q; i += nt) Ls[i * q + k] = df_mul(Ls[i * q + k], inv);
-    __syncthreads();
-    const int r = q - k - 1;
-    for (int idx = tid; idx < r * r; idx += nt) {
-      const int i = k + 1 + idx / r, j = k + 1 + idx % r;
-      if (j <= i) Ls[i * q + j] = df_sub(Ls[i * q + j], df_mul(Ls[i * q + k], Ls[j * q + k]));
+  }
+}
+
+// x = L^-T acc, backward
+__device__ __forceinline__ void warp_solve_upper(const df* L, int ld, const df* dinv, int q, df_acc* acc, df* x) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int s = kStdSlots - 1; s >= 0; --s) {
+    if (32 * s >= q) continue;
+    for (int t = min(q - 32 * s, 32) - 1; t >= 0; --t) {
+      const int k = 32 * s + t;
+      const df xk = shfl_df(df_mul(acc[s].value(), dinv[k]), t);
+      if (lane == t) x[s] = xk;
+      const df nx = df_neg(xk);
+#pragma unroll
+      for (int r = 0; r <= s; ++r) {
+        const int i = lane + 32 * r;
+        if (i < k) acc[r].fma(L[k * ld + i], nx);
+      }
+    }
+  }
+}
+
+// Fallback: H = [[Theta, Ft L^-T], [L^-1 Ft^T, L^-1 Tt L^-T]] with S = L L^T
+// (float-float Cholesky; status = ENOTSPD when S is not positive definite), by
+// one cluster.  Every CTA factors S for itself in its own shared memory (square-root
+// free, one barrier per column: each thread scales by the reciprocal pivot it
+// forms itself; the columns are scaled by 1 / sqrt(d) at the end), which costs
+// less than sending the factor around; the m + q columns of L^-1 [Ft^T | Tt] and
+// then the q columns of L^-1 (L^-1 Tt)^T are solved one warp each over all the
+// CTAs, with a cluster barrier in between.  Bound by the latency of the two chains
+// of q steps.  At m = q = 128 the standard form, back-map and Xc took 3.74 ms of the
+// pencil's 6.6 ms as one block with one thread per column (2.54 + 0.66 + 2 x 0.27 ms
+// of single launches); the pencil is 2.94 ms shorter in this form (0.93 ms at m = 112,
+// q = 72).
+constexpr int kStdCluster = 8;
+constexpr int kStdThreads = 1024;
+
+__global__ void __launch_bounds__(kStdThreads) k_std_form(int m, int q, const double* __restrict__ thg,
+                                                          const df* __restrict__ Ft, const df* __restrict__ Tt,
+                                                          const df* __restrict__ St, df* __restrict__ L, df* Xs,
+                                                          double* H, int* status, const int* skip, int* nfallback) {
+  if (skip && *skip) return;  // every CTA of the cluster returns here alike
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  const int rank = static_cast<int>(cl.block_rank()), CS = static_cast<int>(cl.num_blocks());
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
+  if (rank == 0 && tid == 0 && nfallback) atomicAdd(nfallback, 1);
+  extern __shared__ __align__(16) unsigned char fraw[];
+  const int ld = q | 1;                      // odd row stride: column walks hit different banks
+  df* A = reinterpret_cast<df*>(fraw);       // q x ld
+  df* dinv = A + q * ld;                     // q: 1 / sqrt(d), then 1 / l_kk
+  const long long N = m + q;
+  for (int idx = tid; idx < q * q; idx += nt) A[(idx / q) * ld + idx % q] = St[idx];
+  __syncthreads();
+  int bad = 0;
+  for (int k = 0; k < q; ++k) {
+    df d = A[k * ld + k];
+    if (!(d.hi > 0.f)) {
+      bad = 1;
+      break;  // the same value in every thread of every CTA
+    }
+    const df rinv = df_recip(d);
+    for (int j0 = k + 1; j0 < q; j0 += 32) {
+      const int j = j0 + lane;
+      const df lj = j < q ? df_mul(A[j * ld + k], rinv) : df{0.f, 0.f};
+      for (int i = j0 + warp; i < q; i += nw)
+        if (j <= i) A[i * ld + j] = df_sub(A[i * ld + j], df_mul(A[i * ld + k], lj));
     }
     __syncthreads();
   }
   if (bad) {
-    if (tid == 0 && status) status[0] = AMGEIG_ENOTSPD;
+    if (rank == 0 && tid == 0 && status) status[0] = AMGEIG_ENOTSPD;
     return;
   }
-  for (int idx = tid; idx < q * q; idx += nt) L[idx] = Ls[idx];
-  // Xs = L^-1 Tt (columns in parallel; each thread reads back only what it wrote)
-  for (int c = tid; c < q; c += nt)
-    for (int i = 0; i < q; ++i) {
-      df_acc s = acc_zero();
-      s.add(Tt[i * q + c]);
-      for (int k = 0; k < i; ++k) s.fma(df_neg(Ls[i * q + k]), Xs[k * q + c]);
-      Xs[i * q + c] = df_div(s.value(), Ls[i * q + i]);
-    }
-  __syncthreads();
-  // T = L^-1 Xs^T, written (symmetrised below) into H's lower-right block
-  for (int c = tid; c < q; c += nt)
-    for (int i = 0; i < q; ++i) {
-      df_acc s = acc_zero();
-      s.add(Xs[c * q + i]);
-      for (int k = 0; k < i; ++k) s.fma(df_neg(Ls[i * q + k]), to_df(H[(m + k) * N + m + c]));
-      H[(m + i) * N + m + c] = df_to_double(df_div(s.value(), Ls[i * q + i]));
-    }
-  for (long long idx = tid; idx < static_cast<long long>(m) * m; idx += nt) {
-    const int r = static_cast<int>(idx / m), c = static_cast<int>(idx % m);
-    H[r * N + c] = (r == c) ? thg[r] : 0.0;
-  }
-  // F rows: f_i = L^-1 Ft_i^T
-  for (int r = tid; r < m; r += nt) {
-    df f[kStdMaxQ];
-    for (int i = 0; i < q; ++i) {
-      df_acc s = acc_zero();
-      s.add(Ft[r * q + i]);
-      for (int k = 0; k < i; ++k) s.fma(df_neg(Ls[i * q + k]), f[k]);
-      f[i] = df_div(s.value(), Ls[i * q + i]);
-      const double v = df_to_double(f[i]);
-      H[r * N + m + i] = v;
-      H[(m + i) * N + r] = v;
-    }
-  }
+  for (int k = tid; k < q; k += nt) dinv[k] = df_div(df{1.f, 0.f}, df_sqrt(A[k * ld + k]));
   __syncthreads();
   for (int idx = tid; idx < q * q; idx += nt) {
+    const int i = idx / q, j = idx % q;
+    if (j > i) continue;
+    const df l = df_mul(A[i * ld + j], dinv[j]);  // d_j / sqrt(d_j) on the diagonal
+    A[i * ld + j] = l;
+    if (rank == 0) L[idx] = l;
+  }
+  __syncthreads();
+  for (int k = tid; k < q; k += nt) dinv[k] = df_div(df{1.f, 0.f}, A[k * ld + k]);
+  __syncthreads();
+  df x[kStdSlots];
+  df_acc acc[kStdSlots];
+  for (int c = rank * nw + warp; c < m + q; c += CS * nw) {
+#pragma unroll
+    for (int r = 0; r < kStdSlots; ++r) {
+      const int i = lane + 32 * r;
+      acc[r] = acc_zero();
+      if (i < q) acc[r].add(c < q ? Tt[i * q + c] : Ft[(c - q) * q + i]);
+    }
+    warp_solve_lower(A, ld, dinv, q, acc, x);
+    if (c < q) {
+#pragma unroll
+      for (int r = 0; r < kStdSlots; ++r)
+        if (lane + 32 * r < q) Xs[c * q + lane + 32 * r] = x[r];  // column c of L^-1 Tt
+    } else {
+      const int row = c - q;
+#pragma unroll
+      for (int r = 0; r < kStdSlots; ++r) {
+        const int i = lane + 32 * r;
+        if (i < q) {
+          const double v = df_to_double(x[r]);
+          H[row * N + m + i] = v;
+          H[(m + i) * N + row] = v;
+        }
+      }
+      for (int i = lane; i < m; i += 32) H[row * N + i] = i == row ? thg[row] : 0.0;
+    }
+  }
+  cl.sync();  // L^-1 Tt is complete
+  for (int c = rank * nw + warp; c < q; c += CS * nw) {
+#pragma unroll
+    for (int r = 0; r < kStdSlots; ++r) {
+      const int i = lane + 32 * r;
+      acc[r] = acc_zero();
+      if (i < q) acc[r].add(Xs[i * q + c]);
+    }
+    warp_solve_lower(A, ld, dinv, q, acc, x);
+#pragma unroll
+    for (int r = 0; r < kStdSlots; ++r)
+      if (lane + 32 * r < q) H[(m + lane + 32 * r) * N + m + c] = df_to_double(x[r]);
+  }
+  cl.sync();  // the lower right block is complete: symmetrised in place, one thread per pair
+  for (int idx = rank * nt + tid; idx < q * q; idx += CS * nt) {
     const int a = idx / q, b = idx % q;
     if (b <= a) continue;
     const double v = 0.5 * (H[(m + a) * N + m + b] + H[(m + b) * N + m + a]);
@@ -2557,43 +2628,61 @@ __global__ void __launch_bounds__(512) k_std_form(int m, int q, const double* __
   }
 }
 
-// Fallback back-map: b = L^-T b_std in place (rows m.. of evecs, n x q).
-// b = L^-T b_std for the p wanted columns of evecs ((m + q) x p; L is the border's q x q factor)
-__global__ void k_std_back(int m, int q, int p, const df* __restrict__ L, double* __restrict__ evecs,
-                           const int* skip) {
+// Fallback back-map: b = L^-T b_std in place for the p wanted columns of evecs ((m + q) x p; L is the
+// border's q x q factor), one warp per column.
+constexpr int kBackWarps = 8;
+
+__global__ void __launch_bounds__(32 * kBackWarps) k_std_back(int m, int q, int p, const df* __restrict__ L,
+                                                              double* __restrict__ evecs, const int* skip) {
   if (skip && *skip) return;
-  const int c = threadIdx.x;
+  extern __shared__ __align__(16) unsigned char braw[];
+  df* Ls = reinterpret_cast<df*>(braw);  // q x q (rows are read along them: no padding needed)
+  df* dinv = Ls + q * q;
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
+  for (int idx = tid; idx < q * q; idx += nt)
+    if (idx % q <= idx / q) Ls[idx] = L[idx];
+  for (int k = tid; k < q; k += nt) dinv[k] = df_div(df{1.f, 0.f}, L[k * q + k]);
+  __syncthreads();
+  const int c = blockIdx.x * kBackWarps + (tid >> 5);
   if (c >= p) return;
-  df b[kStdMaxQ];
-  for (int i = q - 1; i >= 0; --i) {
-    df_acc s = acc_zero();
-    s.add(to_df(evecs[(m + i) * static_cast<long long>(p) + c]));
-    for (int k = i + 1; k < q; ++k) s.fma(df_neg(L[k * q + i]), b[k]);
-    b[i] = df_div(s.value(), L[i * q + i]);
+  df x[kStdSlots];
+  df_acc acc[kStdSlots];
+#pragma unroll
+  for (int r = 0; r < kStdSlots; ++r) {
+    const int i = lane + 32 * r;
+    acc[r] = acc_zero();
+    if (i < q) acc[r].add(to_df(evecs[(m + i) * static_cast<long long>(p) + c]));
   }
-  for (int i = 0; i < q; ++i) evecs[(m + i) * static_cast<long long>(p) + c] = df_to_double(b[i]);
+  warp_solve_upper(Ls, q, dinv, q, acc, x);
+#pragma unroll
+  for (int r = 0; r < kStdSlots; ++r) {
+    const int i = lane + 32 * r;
+    if (i < q) evecs[(m + i) * static_cast<long long>(p) + c] = df_to_double(x[r]);
+  }
 }
 
-// Xc = Z_m (a - B b) (d_n x q) and Y = b (q x q) from evecs = [a; b].  Every
-// block forms a - B b in shared memory (b staged there first), then its share
-// of the rows of Xc.
-// Xc = Z_m (a - B b) and Y = b for the columns [j0, j0 + qc) (chunks keep the
-// staged blocks within shared memory when m and q are large)
-// q: the border (columns of V), p: the pairs (columns of evecs, Xc and Y)
-__global__ void __launch_bounds__(kPenThreads) k_xc(int dn, int m, int q, int p, int j0, int qc,
-                                                    const float2* __restrict__ Zdf, const df* __restrict__ KB,
-                                                    const double* __restrict__ evecs, double* __restrict__ Xc,
-                                                    float2* __restrict__ Xc2, double* __restrict__ Y) {
+// Xc = Z_m (a - B b) (d_n x p, also as float-float pairs in Xc2 when non-null) and Y = b (q x p) from
+// evecs = [a; b].  Each block takes kXcCols columns: it stages b, forms a - B b in shared memory and then
+// the d_n rows of the product, so that no work is repeated between blocks.
+// q: the border (columns of V), p: the pairs (columns of evecs, Xc and Y).
+constexpr int kXcCols = 2;
+constexpr int kXcThreads = 512;
+
+__global__ void __launch_bounds__(kXcThreads) k_xc(int dn, int m, int q, int p, const float2* __restrict__ Zdf,
+                                                   const df* __restrict__ KB, const double* __restrict__ evecs,
+                                                   double* __restrict__ Xc, float2* __restrict__ Xc2,
+                                                   double* __restrict__ Y) {
   extern __shared__ __align__(16) unsigned char xraw[];
-  df* bs = reinterpret_cast<df*>(xraw);  // q x qc: b[:, j0:j0+qc]
-  df* tmp = bs + q * qc;                 // m x qc
+  const int j0 = blockIdx.x * kXcCols, qc = min(kXcCols, p - j0);
+  df* bs = reinterpret_cast<df*>(xraw);  // q x kXcCols: b[:, j0:j0+qc]
+  df* tmp = bs + q * kXcCols;            // m x kXcCols
   const int tid = threadIdx.x, nt = blockDim.x;
   const int q2 = 2 * q;
   for (int idx = tid; idx < q * qc; idx += nt) {
     const int r = idx / qc, jj = idx % qc;
     const double v = evecs[static_cast<long long>(m + r) * p + j0 + jj];
-    bs[idx] = to_df(v);
-    if (blockIdx.x == 0) Y[r * p + j0 + jj] = v;
+    bs[r * kXcCols + jj] = to_df(v);
+    Y[r * p + j0 + jj] = v;
   }
   __syncthreads();
   for (int idx = tid; idx < m * qc; idx += nt) {
@@ -2605,31 +2694,29 @@ __global__ void __launch_bounds__(kPenThreads) k_xc(int dn, int m, int q, int p,
     int t = 0;
 #pragma unroll 4
     for (; t + 4 <= q; t += 4) {
-      c0.fma(Bi[t], bs[t * qc + jj]);
-      c1.fma(Bi[t + 1], bs[(t + 1) * qc + jj]);
-      c2.fma(Bi[t + 2], bs[(t + 2) * qc + jj]);
-      c3.fma(Bi[t + 3], bs[(t + 3) * qc + jj]);
+      c0.fma(Bi[t], bs[t * kXcCols + jj]);
+      c1.fma(Bi[t + 1], bs[(t + 1) * kXcCols + jj]);
+      c2.fma(Bi[t + 2], bs[(t + 2) * kXcCols + jj]);
+      c3.fma(Bi[t + 3], bs[(t + 3) * kXcCols + jj]);
     }
-    for (; t < q; ++t) c0.fma(Bi[t], bs[t * qc + jj]);
+    for (; t < q; ++t) c0.fma(Bi[t], bs[t * kXcCols + jj]);
     c0.merge(c1);
     c2.merge(c3);
     c0.merge(c2);
-    tmp[idx] = df_sub(to_df(evecs[static_cast<long long>(i) * p + j0 + jj]), c0.value());
+    tmp[i * kXcCols + jj] = df_sub(to_df(evecs[static_cast<long long>(i) * p + j0 + jj]), c0.value());
   }
   __syncthreads();
-  const int rows = (dn + gridDim.x - 1) / gridDim.x;
-  const int r0 = blockIdx.x * rows, r1 = min(dn, r0 + rows);
-  for (int idx = tid; idx < (r1 - r0) * qc; idx += nt) {
-    const int l = r0 + idx / qc, jj = idx % qc;
+  for (int idx = tid; idx < dn * qc; idx += nt) {
+    const int l = idx / qc, jj = idx % qc;
     const float2* zl = Zdf + static_cast<long long>(l) * dn;
     df_acc s0 = acc_zero(), s1 = acc_zero();
     int i = 0;
 #pragma unroll 8
     for (; i + 2 <= m; i += 2) {  // unrolled: the row's loads (L2) in flight together
-      s0.fma(to_df(zl[i]), tmp[i * qc + jj]);
-      s1.fma(to_df(zl[i + 1]), tmp[(i + 1) * qc + jj]);
+      s0.fma(to_df(zl[i]), tmp[i * kXcCols + jj]);
+      s1.fma(to_df(zl[i + 1]), tmp[(i + 1) * kXcCols + jj]);
     }
-    if (i < m) s0.fma(to_df(zl[i]), tmp[i * qc + jj]);
+    if (i < m) s0.fma(to_df(zl[i]), tmp[i * kXcCols + jj]);
     s0.merge(s1);
     const df v = s0.value();
     Xc[static_cast<long long>(l) * p + j0 + jj] = df_to_double(v);
@@ -3043,16 +3130,14 @@ void launch_pencil_solve(PencilWork* w, int dn, int m, int q, const double* C64,
   const size_t srs = sizeof(df) * (2.0 * m + 2.0 * m * q + 3.0 * q * q + 2.0 * q + 2.0 * n);
   const size_t chs = sizeof(df) * (1.0 * n * q + 5.0 * q * q + 2.0 * m + 1.0 * m * q + 1.0 * q * (q + kMaxCluster) +
                                     3.0 * n * kMaxCluster + 1.0 * kMaxCluster * q);
-  const size_t fs = sizeof(df) * q * q;
+  const size_t fs = sizeof(df) * (static_cast<size_t>(q) * (q | 1) + q);
+  const size_t bks = sizeof(df) * (static_cast<size_t>(q) * q + q);
+  const size_t xsc = sizeof(df) * static_cast<size_t>(m + q) * kXcCols;
   // the structured iteration finds one pair per border column: a wider border (p < q) takes the dense path
   const bool fast = p == q && q <= kSrqiMaxQ && srs <= 200 * 1024 && chs <= 220 * 1024;
-  // Xc = Z_m (a - B b) runs in column chunks whose staged blocks fit in 200 KB
-  const int qc = static_cast<int>(std::max<size_t>(
-      1, std::min<size_t>(p, (200 * 1024) / (sizeof(df) * static_cast<size_t>(m + q)))));
-  const int nxc = (p + qc - 1) / qc;
   // kernels launched here; the dense eigensolver's launcher counts its own
   ProfScope ps(st, P_PENCIL, 8.0 * (2.0 * dn * m + 2.0 * dn * q + 2.0 * m * q + 3.0 * q * q + 1.0 * n * q), 0.0,
-               (fast ? 6 : 4) + nxc);
+               fast ? 7 : 5);
   if (Cdf) {
     smem_attr((const void*)k_kb<float2>, kbs);
     k_kb<float2><<<2 * q, kPenThreads, kbs, st>>>(dn, m, q, Zdf, Cdf, w->KB);
@@ -3073,16 +3158,28 @@ void launch_pencil_solve(PencilWork* w, int dn, int m, int q, const double* C64,
     skip = w->sr_flag;
   }
   smem_attr((const void*)k_std_form, fs);
-  k_std_form<<<1, 512, fs, st>>>(m, q, theta, w->Ft, w->Tt, w->St, w->Lq, w->Xq, w->H, status, skip, nfallback);
-  launch_syev_df(w, n, p, w->H, mu, w->Yh, st, skip);
-  k_std_back<<<1, kStdMaxQ, 0, st>>>(m, q, p, w->Lq, w->Yh, skip);
-  // Xc = Z_m (a - B b), Y = b
-  for (int j0 = 0; j0 < p; j0 += qc) {
-    const int wc = std::min(qc, p - j0);
-    const size_t xsc = sizeof(df) * static_cast<size_t>(m + q) * wc;
-    smem_attr((const void*)k_xc, xsc);
-    k_xc<<<64, kPenThreads, xsc, st>>>(dn, m, q, p, j0, wc, Zdf, w->KB, w->Yh, Xc, Xcdf, Y);
+  {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kStdCluster);
+    cfg.blockDim = dim3(kStdThreads);
+    cfg.dynamicSmemBytes = fs;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = kStdCluster;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, k_std_form, m, q, theta, static_cast<const df*>(w->Ft), static_cast<const df*>(w->Tt),
+                       static_cast<const df*>(w->St), w->Lq, w->Xq, w->H, status, skip, nfallback);
   }
+  launch_syev_df(w, n, p, w->H, mu, w->Yh, st, skip);
+  smem_attr((const void*)k_std_back, bks);
+  k_std_back<<<ceil_div(p, kBackWarps), 32 * kBackWarps, bks, st>>>(m, q, p, w->Lq, w->Yh, skip);
+  // Xc = Z_m (a - B b), Y = b
+  smem_attr((const void*)k_xc, xsc);
+  k_xc<<<ceil_div(p, kXcCols), kXcThreads, xsc, st>>>(dn, m, q, p, Zdf, w->KB, w->Yh, Xc, Xcdf, Y);
 }
 
 void launch_mass_factor(PencilWork* w, int dn, const double* Mn, int* status, cudaStream_t st) {
