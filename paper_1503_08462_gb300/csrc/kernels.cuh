@@ -22,7 +22,8 @@ struct DevCsr {
   __nv_bfloat16* vbf = nullptr;  // v64 rounded to bfloat16 (the V-cycle's operators, AMGEIG_MIXED_BF16)
   // launch shape of the float32 V-cycle kernels on this operator, per block width in float4
   // columns w4 <= 32, chosen by the autotuner: (log2 streams) << 5 | (log2 column lanes per
-  // stream) << 2 | columns per lane; 0 = not tuned (the rule applies)
+  // stream) << 2 | columns per lane; 128 = one block per row (smoothing sweeps); 0 = not tuned (the
+  // rule applies)
   unsigned char tuned[33] = {};
 };
 

@@ -291,12 +291,18 @@ struct F4Geo {
   int G, cpt;
   int S = 1;  // nonzero streams per row: the row's G lanes form S groups of G / S column lanes, group k
               // takes the nonzeros p0 + k, p0 + k + S, ... and the groups' sums are added at the end
+  // cpt = 0: one block of G = S * w4 threads per row (k_smooth_row), S streams of w4 lanes
 };
+
+// Streams of the block-per-row layout: blocks of 96-256 threads.
+int row_streams(int w4) { return w4 <= 8 ? 32 : w4 <= 16 ? 16 : 8; }
+// Whether a level's rows are long enough for it (see k_smooth_row)
+bool row_layout(long long rows, long long nnz) { return nnz >= 96 * rows && rows < 65536; }
 
 // Few lanes per row pay off only while the rows alone keep the GPU full: below
 // about four resident waves of row groups the one-column-per-lane layout (more
 // threads, shorter chains) is faster on the coarse levels.
-F4Geo f4_geo(int w4, long long rows, long long nnz = 0) {
+F4Geo f4_geo(int w4, long long rows, long long nnz, bool sweep) {
   int G = 1;
   while (G * 3 < w4 && G < 32) G <<= 1;
   int cpt = (w4 + G - 1) / G;
@@ -304,6 +310,7 @@ F4Geo f4_geo(int w4, long long rows, long long nnz = 0) {
     G <<= 1;
     cpt = (w4 + G - 1) / G;
   }
+  if (sweep && w4 <= 32 && row_layout(rows, nnz)) return F4Geo{w4 * row_streams(w4), 0, row_streams(w4)};
   if (rows * G < 4LL * kNumSms * 1024) {
     G = 1;
     while (G < w4 && G < 32) G <<= 1;
@@ -319,15 +326,18 @@ F4Geo f4_geo(int w4, long long rows, long long nnz = 0) {
   return F4Geo{G, cpt, 1};
 }
 
-// the operator's tuned shape at this width, else the rule
-F4Geo geo_of(const DevCsr& S, int w4) {
+// the operator's tuned shape at this width, else the rule (sweep: a smoothing sweep, which has the
+// block-per-row layout)
+F4Geo geo_of(const DevCsr& S, int w4, bool sweep) {
   if (w4 >= 1 && w4 <= 32 && S.tuned[w4]) {
     const int v = S.tuned[w4];
-    // tuned: column lanes per stream (log2, bits 2-4), columns per lane (bits 0-1), streams (log2, bits 5-6)
+    // tuned: column lanes per stream (log2, bits 2-4), columns per lane (bits 0-1), streams (log2, bits 5-6);
+    // bit 7: the block-per-row layout
+    if (v & 128) return F4Geo{w4 * row_streams(w4), 0, row_streams(w4)};
     const int streams = 1 << ((v >> 5) & 3);
     return F4Geo{(1 << ((v >> 2) & 7)) * streams, v & 3, streams};
   }
-  return f4_geo(w4, S.rows, S.nnz);
+  return f4_geo(w4, S.rows, S.nnz, sweep);
 }
 
 __device__ __forceinline__ void fma4(float s, const float4& x, float4& acc) {
@@ -354,6 +364,54 @@ __device__ __forceinline__ void reduce_streams(float4 (&acc)[CPT], int S, int gs
       acc[t].y += __shfl_down_sync(0xffffffffu, acc[t].y, o);
       acc[t].z += __shfl_down_sync(0xffffffffu, acc[t].z, o);
       acc[t].w += __shfl_down_sync(0xffffffffu, acc[t].w, o);
+    }
+  }
+}
+
+// The results of one float4 column c4 of one row from its sum acc = (A x)_row (MODE 0: (A D^-1 b)_row).
+template <int MODE>
+__device__ __forceinline__ void smooth_store(float4 acc, int row, int c4, int w4, float di,
+                                             const float4* __restrict__ b, const float4* __restrict__ x,
+                                             float4* __restrict__ out1, float4* __restrict__ out2,
+                                             const double* __restrict__ U, double* __restrict__ V, int qv,
+                                             const float2* __restrict__ U2, float2* __restrict__ V2,
+                                             const float4* __restrict__ xadd) {
+  const long long o = static_cast<long long>(row) * w4 + c4;
+  const float4 bi = b[o];
+  const float4 res = make_float4(bi.x - acc.x, bi.y - acc.y, bi.z - acc.z, bi.w - acc.w);
+  if (MODE == 0) {
+    out1[o] = make_float4(di * bi.x, di * bi.y, di * bi.z, di * bi.w);
+    out2[o] = res;
+  } else if (MODE == 2) {
+    out1[o] = res;
+  } else {
+    const float4 xi = x[o];
+    const float4 xn = make_float4(fmaf(di, res.x, xi.x), fmaf(di, res.y, xi.y), fmaf(di, res.z, xi.z),
+                                  fmaf(di, res.w, xi.w));
+    if (MODE == 1) {
+      out1[o] = xn;
+    } else if (MODE == 3) {
+      const long long vb = static_cast<long long>(row) * qv + 4 * c4;
+      const float xs[4] = {xn.x, xn.y, xn.z, xn.w};
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (4 * c4 + k < qv) V[vb + k] = U[vb + k] + static_cast<double>(xs[k]);
+    } else {
+      // MODE 4: float-float V = U + x (+ xadd: the earlier V-cycles' sum)
+      const long long vb = static_cast<long long>(row) * qv + 4 * c4;
+      float4 xt = xn;
+      if (xadd) {
+        const float4 e = xadd[o];
+        xt = make_float4(xn.x + e.x, xn.y + e.y, xn.z + e.z, xn.w + e.w);
+      }
+      const float xs[4] = {xt.x, xt.y, xt.z, xt.w};
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (4 * c4 + k < qv) {
+          const float2 u = U2[vb + k];
+          const df r = df_add(df{u.x, u.y}, df{xs[k], 0.f});
+          V2[vb + k] = make_float2(r.hi, r.lo);
+        }
     }
   }
 }
@@ -399,46 +457,71 @@ __global__ void __launch_bounds__(kThreads, 6) k_smooth_f4(int n, const int* __r
 #pragma unroll
   for (int t = 0; t < CPT; ++t) {
     const int c4 = lane + t * gs;
-    if (c4 >= w4) continue;
-    const long long o = static_cast<long long>(row) * w4 + c4;
-    const float4 bi = b[o];
-    const float4 res = make_float4(bi.x - acc[t].x, bi.y - acc[t].y, bi.z - acc[t].z, bi.w - acc[t].w);
-    if (MODE == 0) {
-      out1[o] = make_float4(di * bi.x, di * bi.y, di * bi.z, di * bi.w);
-      out2[o] = res;
-    } else if (MODE == 2) {
-      out1[o] = res;
-    } else {
-      const float4 xi = x[o];
-      const float4 xn = make_float4(fmaf(di, res.x, xi.x), fmaf(di, res.y, xi.y), fmaf(di, res.z, xi.z),
-                                    fmaf(di, res.w, xi.w));
-      if (MODE == 1) {
-        out1[o] = xn;
-      } else if (MODE == 3) {
-        const long long vb = static_cast<long long>(row) * qv + 4 * c4;
-        const float xs[4] = {xn.x, xn.y, xn.z, xn.w};
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-          if (4 * c4 + k < qv) V[vb + k] = U[vb + k] + static_cast<double>(xs[k]);
-      } else {
-        // MODE 4: float-float V = U + x (+ xadd: the earlier V-cycles' sum)
-        const long long vb = static_cast<long long>(row) * qv + 4 * c4;
-        float4 xt = xn;
-        if (xadd) {
-          const float4 e = xadd[o];
-          xt = make_float4(xn.x + e.x, xn.y + e.y, xn.z + e.z, xn.w + e.w);
-        }
-        const float xs[4] = {xt.x, xt.y, xt.z, xt.w};
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-          if (4 * c4 + k < qv) {
-            const float2 u = U2[vb + k];
-            const df r = df_add(df{u.x, u.y}, df{xs[k], 0.f});
-            V2[vb + k] = make_float2(r.hi, r.lo);
-          }
-      }
-    }
+    if (c4 < w4) smooth_store<MODE>(acc[t], row, c4, w4, di, b, x, out1, out2, U, V, qv, U2, V2, xadd);
   }
+}
+
+// The same sweep with one block per row, for the coarse levels whose rows are
+// long: the Galerkin operators of 3D problems keep 200-600 nonzeros a row at a
+// few thousand rows, where a warp per row leaves chains of 50-150 dependent
+// gathers and most of the chip idle.  The block's threads are S streams of exactly w4
+// column lanes (no idle lanes at widths that are not powers of two), stream k
+// takes the nonzeros k, k + S, ..., four gathers in flight per thread, and the
+// streams' sums meet in shared memory in a fixed tree.  Bound by the gathers'
+// L2 latency and rate.  Cube of 250,047 unknowns, 20 columns (event times, a warp per
+// row -> a block per row): 5494 rows of 361 nonzeros 53.5 -> 22.9 us, 2471 x 524 70.9 -> 18.5,
+// 1142 x 598 64.1 -> 13.7, 521 x 469 39.9 -> under 12; 12,620 x 214 38.8 -> 33.4; rows
+// below ~100 nonzeros gain nothing, which is where the rule's line lies (the tuner times both).
+template <int MODE, typename TV>
+__global__ void __launch_bounds__(256) k_smooth_row(int n, const int* __restrict__ rp, const int* __restrict__ ci,
+                                                    const TV* __restrict__ a, const float* __restrict__ dinv,
+                                                    const float4* __restrict__ b, const float4* __restrict__ x, int w4,
+                                                    float4* __restrict__ out1, float4* __restrict__ out2,
+                                                    const double* __restrict__ U, double* __restrict__ V, int qv,
+                                                    int S, const float2* __restrict__ U2, float2* __restrict__ V2,
+                                                    const float4* __restrict__ xadd) {
+  __shared__ float4 part[256];
+  const int row = blockIdx.x;
+  const int sub = threadIdx.x / w4, lane = threadIdx.x - sub * w4;
+  const int p1 = rp[row + 1];
+  const float4* src = (MODE == 0 ? b : x) + lane;
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  int p = rp[row] + sub;
+  for (; p + 3 * S < p1; p += 4 * S) {
+    int j[4];
+    float s[4];
+    float4 v[4];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      j[t] = ci[p + t * S];
+      s[t] = to_f(a[p + t * S]);
+    }
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      v[t] = src[static_cast<long long>(j[t]) * w4];
+      if (MODE == 0) s[t] *= dinv[j[t]];
+    }
+#pragma unroll
+    for (int t = 0; t < 4; ++t) fma4(s[t], v[t], acc);
+  }
+  for (; p < p1; p += S) {
+    const int j = ci[p];
+    float s = to_f(a[p]);
+    if (MODE == 0) s *= dinv[j];
+    fma4(s, src[static_cast<long long>(j) * w4], acc);
+  }
+  part[threadIdx.x] = acc;
+  __syncthreads();
+  for (int o = S >> 1; o > 0; o >>= 1) {
+    if (sub < o) {
+      const float4 u = part[threadIdx.x + o * w4];
+      acc = make_float4(acc.x + u.x, acc.y + u.y, acc.z + u.z, acc.w + u.w);
+      part[threadIdx.x] = acc;
+    }
+    __syncthreads();
+  }
+  if (sub == 0)
+    smooth_store<MODE>(acc, row, lane, w4, dinv ? dinv[row] : 0.f, b, x, out1, out2, U, V, qv, U2, V2, xadd);
 }
 
 template <int CPT, typename TV>
@@ -488,7 +571,20 @@ template <int MODE>
 void smooth_f4(const DevCsr& A, const float* dinv, const float* b, const float* x, int w4, float* out1, float* out2,
                const double* U, double* V, int qv, const float2* U2, float2* V2, const float* xadd,
                cudaStream_t st, bool bf16 = false, const F4Geo* force = nullptr) {
-  const F4Geo g = force ? *force : geo_of(A, w4);
+  const F4Geo g = force ? *force : geo_of(A, w4, true);
+  if (g.cpt == 0) {
+#define AMGEIG_SMOOTH_ROW(TV, VALS)                                                                              \
+  k_smooth_row<MODE, TV><<<A.rows, g.G, 0, st>>>(                                                                \
+      A.rows, A.rp, A.ci, VALS, dinv, reinterpret_cast<const float4*>(b), reinterpret_cast<const float4*>(x), w4, \
+      reinterpret_cast<float4*>(out1), reinterpret_cast<float4*>(out2), U, V, qv, g.S, U2, V2,                   \
+      reinterpret_cast<const float4*>(xadd))
+    if (bf16)
+      AMGEIG_SMOOTH_ROW(__nv_bfloat16, A.vbf);
+    else
+      AMGEIG_SMOOTH_ROW(float, A.v32);
+#undef AMGEIG_SMOOTH_ROW
+    return;
+  }
   const int blocks = ceil_div(A.rows, kThreads / g.G);
 #define AMGEIG_SMOOTH_T(C, TV, VALS)                                                                         \
   k_smooth_f4<MODE, C, TV><<<blocks, kThreads, 0, st>>>(                                                       \
@@ -812,7 +908,7 @@ void launch_spmm_f32(const DevCsr& S, const float* X, int width, float* Y, bool 
     return;
   }
   const int w4 = width / 4;
-  const F4Geo g = geo_of(S, w4);
+  const F4Geo g = geo_of(S, w4, false);
   spmm_f4_geo(S, X, w4, Y, accumulate, st, bf16, g);
 }
 
@@ -1090,7 +1186,7 @@ void launch_composite_rows(const DevCsr& P, const int* nrp, const int* nci, cons
 TuneResult autotune_f4(DevCsr& S, int kind, int w4, const float* dinv, const float* x, const float* b, float* out,
                        cudaStream_t st) {
   TuneResult r;
-  const F4Geo rule = f4_geo(w4, S.rows, S.nnz);
+  const F4Geo rule = f4_geo(w4, S.rows, S.nnz, kind == 0);
   r.rule_G = rule.G;
   r.rule_cpt = rule.cpt;
   r.S = rule.S;
@@ -1137,9 +1233,24 @@ TuneResult autotune_f4(DevCsr& S, int kind, int w4, const float* dinv, const flo
         r.S = streams;
       }
     }
+  // and, for the smoothing sweeps, the block-per-row layout where a row has a nonzero for every stream
+  bool by_row = false;
+  if (kind == 0 && S.nnz >= static_cast<long long>(row_streams(w4)) * S.rows) {
+    const F4Geo g{w4 * row_streams(w4), 0, row_streams(w4)};
+    const float us = time_us(g);
+    if (us < best) {
+      best = us;
+      r.G = g.G;
+      r.cpt = g.cpt;
+      r.S = g.S;
+      by_row = true;
+    }
+  }
   r.us = best;
   r.rule_us = time_us(rule);
-  if (r.G > 0 && cudaGetLastError() == cudaSuccess) {
+  if (by_row && cudaGetLastError() == cudaSuccess) {
+    S.tuned[w4] = 128;
+  } else if (r.G > 0 && cudaGetLastError() == cudaSuccess) {
     int lg = 0, ls = 0;
     while ((1 << lg) < r.G / r.S) ++lg;
     while ((1 << ls) < r.S) ++ls;
