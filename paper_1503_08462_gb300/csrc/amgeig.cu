@@ -928,6 +928,19 @@ int correction_tail_krylov(amgeig_hierarchy_t* h, SolveWork* w, int k, const amg
   return AMGEIG_OK;
 }
 
+// Whether the recombination applies the composite prolongation I_n^k in one pass rather than the chain
+// P_k ... P_{n-2}.  The composite costs one compensated product per nonzero and column, the chain its
+// own (fewer) nonzeros, the intermediate blocks' traffic and a launch per level.  In 2D the composite has
+// ~1.8 times the chain's nonzeros and wins (one pass, nothing stored between); in 3D its rows fill up
+// (cube of 250,047 unknowns, 17 columns: ~25 M nonzeros against 1.6 M) and the chain wins: 465 us per
+// correction with the composite, 210 with the chain (132 of transfers, 78 of V Y).  Small levels keep
+// the single launch.
+bool composite_pays(const amgeig_hierarchy_t* h, int k) {
+  long long chain = 0;
+  for (int l = k; l + 1 < h->nlev; ++l) chain += h->P[l].nnz;
+  return h->sizes[k] < 8192 || h->PC[k].nnz <= 4 * chain;
+}
+
 int correction_tail(amgeig_hierarchy_t* h, SolveWork* w, int k, const amgeig_options& o, cudaStream_t st) {
   if (o.krylov == 2) return correction_tail_krylov(h, w, k, o, st);
   const int q = w->qt;
@@ -965,7 +978,7 @@ int correction_tail(amgeig_hierarchy_t* h, SolveWork* w, int k, const amgeig_opt
     }
     launch_pencil_solve(w->pw, h->dn, modes, q, nullptr, cur, w->G, h->Zdf, h->theta, w->mu, w->Xc,
                         as_df(w->PX[n - 1]), w->Yv, h->dstatus, st, w->nfallback);
-    if (q <= 32) {
+    if (q <= 32 && composite_pays(h, k)) {
       // U = I_n^k Xc + V Y in one pass: the composite prolongation is applied row by row
       const DevCsr& PC = h->PC[k];
       launch_recombine_pc_df(Nk, PC.nnz, PC.rp, PC.ci, PC.d2, as_df(w->PX[n - 1]), as_df(w->V), w->Yv, q,

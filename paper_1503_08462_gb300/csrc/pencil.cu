@@ -761,7 +761,10 @@ __device__ void syev_group_rr(int G, const df* Z, long long ldz, const df* dd, c
       }
     }
   }
-  // order eigenvalues ascending (selection by rank; ties broken by index)
+  // order eigenvalues ascending (selection by rank; ties broken by index); the identity first, so that
+  // perm holds valid columns even when a NaN leaves ranks unassigned
+  for (int j = tid; j < G; j += nt) perm[j] = j;
+  __syncthreads();
   for (int j = tid; j < G; j += nt) {
     const df lj = Hq[j * G + j];
     int rank = 0;
