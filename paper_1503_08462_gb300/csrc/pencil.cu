@@ -36,6 +36,7 @@
 #include <cstdio>
 #include <map>
 #include <mutex>
+#include <type_traits>
 
 #include "common.cuh"
 #include "kernels.cuh"
@@ -87,6 +88,10 @@ struct PencilWork {
 namespace {
 
 // ------------------------------------------------------------ block helpers
+
+__device__ __forceinline__ df shfl_df(df v, int src) {
+  return df{__shfl_sync(0xffffffffu, v.hi, src), __shfl_sync(0xffffffffu, v.lo, src)};
+}
 
 // sum_i a[i sa] b[i sb] (i < len) in float-float with four interleaved
 // accumulators: independent chains keep the float32 pipes busy in these
@@ -150,13 +155,10 @@ __device__ __forceinline__ int sturm_count_df(const df* dd, const df* ee2, int n
 
 // ------------------------------------------------------------ float-float syev
 //
-// The phases of the solver are device functions with two drivers: k_syev_df
-// runs all of them in one block (the allocation-free entry point), the split
-// path runs the tridiagonalisation in one block (k_syev_tri) and spreads the
-// per-eigenvalue phases over many: the shifts one warp each (k_syev_vals),
-// inverse iteration and clean-up one block per group of close shifts
-// (k_syev_vecs) and the back-transformation one warp per eigenvector
-// (k_syev_back).  Each eigenvalue's phases do the same arithmetic on both.
+// Four kernels: the tridiagonalisation (k_syev_tri, one block, or k_syev_tri_cl,
+// a cluster of 16), the shifts (k_syev_vals), inverse iteration and clean-up
+// one block per group of close shifts (k_syev_vecs) and the
+// back-transformation (k_syev_back).
 
 // Householder tridiagonalisation of the symmetric W (n x n, row stride LD,
 // full storage) by the whole block.  Four barriers per step: the norm of the
@@ -308,18 +310,7 @@ __device__ void syev_bounds(const float* sd, const float* se2, int n, float* sf)
   sf[3] = fmaxf(1.0e-30f, 1.0e-35f * fmaxf(emax2, 1.f));
 }
 
-// float32 bisection for the (j+1)-th smallest eigenvalue, one thread.
-__device__ float syev_bisect(int j, const float* sd, const float* se2, int n, float gl, float gu, float pivmin) {
-  float lo = gl, hi = gu;
-  for (int it = 0; it < 80; ++it) {
-    const float mid = 0.5f * (lo + hi);
-    if (mid <= lo || mid >= hi) break;
-    if (sturm_count(sd, se2, n, mid, pivmin) > j) hi = mid; else lo = mid;
-  }
-  return 0.5f * (lo + hi);
-}
-
-// The same bracket by one warp: 32-point multisection, 33x narrower per round
+// float32 bracket of the (j+1)-th smallest eigenvalue by one warp: 32-point multisection, 33x narrower per round
 // (Golub & Van Loan 8.4.1), until the float32 points stop separating.
 __device__ float syev_multisect(int j, const float* sd, const float* se2, int n, float gl, float gu, float pivmin) {
   const int lane = threadIdx.x & 31;
@@ -385,39 +376,6 @@ __device__ df syev_refine_shift(int j, float s0, const df* dd, const df* ee2, in
 // cluster and group thresholds below.
 __device__ __forceinline__ float shift_gap(const df* shd, int j) {
   return j > 0 ? df_float(df_sub(shd[j], shd[j - 1])) : 3.0e38f;
-}
-
-// Clusters and clean-up groups of the ascending shifts, by one thread.  Shifts
-// closer than 1e-9 ||T|| form clusters, iterated in rounds with Gram-Schmidt
-// (cpos[j]: position of j in its cluster, which starts at cstart[j]); runs of
-// shifts closer than 1e-4 ||T|| form the groups [gs0[j], gs1[j]) of the
-// Rayleigh-Ritz clean-up.  si[0] = the largest cluster position, si[1] = 1 if
-// any two shifts are closer than 1e-4 ||T||.
-__device__ void syev_groups(const df* shd, int nwant, float tnorm, float pivmin, int* cstart, int* cpos, int* gs0,
-                            int* gs1, int* si) {
-  const float ctol = 1.0e-9f * tnorm + pivmin, rtol = 1.0e-4f * tnorm;
-  int maxpos = 0, close = 0, gstart = 0;
-  for (int j = 0; j < nwant; ++j) {
-    const float gap = shift_gap(shd, j);
-    if (gap <= ctol) {
-      cstart[j] = cstart[j - 1];
-      cpos[j] = cpos[j - 1] + 1;
-    } else {
-      cstart[j] = j;
-      cpos[j] = 0;
-    }
-    if (gap <= rtol) {
-      close = 1;
-    } else if (j > 0) {
-      for (int i = gstart; i < j; ++i) gs1[i] = j;
-      gstart = j;
-    }
-    gs0[j] = gstart;
-    maxpos = max(maxpos, cpos[j]);
-  }
-  for (int i = gstart; i < nwant; ++i) gs1[i] = nwant;
-  si[0] = maxpos;
-  si[1] = close;
 }
 
 // Inverse iteration in float-float for the shift sg of index j, one thread:
@@ -796,189 +754,6 @@ __device__ void syev_group_rr(int G, const df* Z, long long ldz, const df* dd, c
   __syncthreads();
 }
 
-// ---- one-block driver
-//
-// Dynamic shared memory: v, p (df, n each), sd, se2 (float, n each), shift
-// (float, nwant), cstart, cpos (int, nwant), d, e, tau, e^2 (df, n each),
-// shifts (df, nwant), gs0, gs1 (int, nwant), then -- when they fit -- the
-// working matrix W (n x ldw df), the inverse-iteration factors (2 x n x nwant
-// df) and the tridiagonal eigenvectors Zt (n x nwant df).  `flags` bit 0/1/2
-// says which of W / factors / Zt live in shared memory; the others use the
-// global workspace (same layout), so one code path serves every size.
-constexpr int kSyW = 1, kSyF = 2, kSyZ = 4;
-
-__global__ void __launch_bounds__(kSyThreads) k_syev_df(int n, int nwant, int ldw, int flags,
-                                                        const double* __restrict__ H, double* __restrict__ evals,
-                                                        double* __restrict__ evecs, df* __restrict__ Wg,
-                                                        df* __restrict__ tau_g, df* __restrict__ dd_g,
-                                                        df* __restrict__ ee_g, df* __restrict__ facg,
-                                                        df* __restrict__ Ztg, df* __restrict__ rrw,
-                                                        int* __restrict__ perm, const int* __restrict__ skip) {
-  if (skip != nullptr && *skip != 0) return;  // the structured fast path already produced the pairs
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  df* v = reinterpret_cast<df*>(smem_raw);
-  df* p = v + n;
-  float* sd = reinterpret_cast<float*>(p + n);
-  float* se2 = sd + n;
-  float* shift = se2 + n;
-  int* cstart = reinterpret_cast<int*>(shift + nwant);
-  int* cpos = cstart + nwant;
-  size_t off = (2 * sizeof(df) * n + 2 * sizeof(float) * n + sizeof(float) * nwant + 2 * sizeof(int) * nwant +
-                4 * sizeof(df) * n + sizeof(df) * nwant + 2 * sizeof(int) * nwant + 15) &
-               ~static_cast<size_t>(15);
-  df* W = Wg;
-  if (flags & kSyW) {
-    W = reinterpret_cast<df*>(smem_raw + off);
-    off += sizeof(df) * static_cast<size_t>(n) * ldw;
-  }
-  df* fac = facg;
-  if (flags & kSyF) {
-    fac = reinterpret_cast<df*>(smem_raw + off);
-    off += sizeof(df) * 2 * static_cast<size_t>(n) * nwant;
-  }
-  df* Zt = Ztg;
-  if (flags & kSyZ) Zt = reinterpret_cast<df*>(smem_raw + off);
-  __shared__ df_acc red[32];
-  __shared__ float sf[4];
-  __shared__ int si[4];
-
-  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
-  const long long N = n, LD = ldw;
-  // the tridiagonal (d, e) and the Householder scalars live in shared memory
-  df* dd = reinterpret_cast<df*>(cpos + nwant);
-  df* ee = dd + n;
-  df* tau = ee + n;
-  df* ee2 = tau + n;     // e_i^2 in float-float (Sturm counts)
-  df* shd = ee2 + n;     // float-float shifts (nwant)
-  int* gs0 = reinterpret_cast<int*>(shd + nwant);  // clean-up group [gs0[j], gs1[j]) of index j
-  int* gs1 = gs0 + nwant;
-  __shared__ df_acc red_sig[32], red_vp[32];
-
-  for (long long i = tid; i < N * N; i += nt) W[(i / N) * LD + (i % N)] = df_from_double(H[i]);
-  __syncthreads();
-  syev_tridiagonalise(n, W, LD, v, p, dd, ee, tau, red_sig, red_vp, nullptr);
-
-  // ---- bisection (float32) for the nwant smallest eigenvalues, refined in float-float
-  for (int i = tid; i < n; i += nt) {
-    sd[i] = df_float(dd[i]);
-    if (i + 1 < n) {
-      const float e = df_float(ee[i]);
-      se2[i] = e * e;
-    }
-  }
-  __syncthreads();
-  if (tid == 0) syev_bounds(sd, se2, n, sf);
-  __syncthreads();
-  const float gl = sf[0], gu = sf[1], tnorm = sf[2], pivmin = sf[3];
-  for (int j = tid; j < nwant; j += nt) shift[j] = syev_bisect(j, sd, se2, n, gl, gu, pivmin);
-  for (int i = tid; i + 1 < n; i += nt) ee2[i] = df_mul(ee[i], ee[i]);
-  __syncthreads();
-  for (int j = warp; j < nwant; j += nw) {
-    const df s = syev_refine_shift(j, shift[j], dd, ee2, n, gl, gu, tnorm, pivmin);
-    if (lane == 0) shd[j] = s;
-  }
-  __syncthreads();
-  if (tid == 0) syev_groups(shd, nwant, tnorm, pivmin, cstart, cpos, gs0, gs1, si);
-  __syncthreads();
-  const int maxpos = si[0];
-  const bool cleanup = si[1] != 0;
-
-  // ---- inverse iteration in float-float: T - s I = L D L^T -----------------
-  // factor arrays (element i of eigen-index j at [i * nwant + j]):
-  //   fac[0 .. n*nwant) = 1/d_i, fac[n*nwant .. 2n*nwant) = l_i
-  const long long NW = nwant;
-  const df pv = df{fmaxf(3.6e-15f * tnorm, 1.0e-30f), 0.f};
-  for (int round = 0; round <= maxpos; ++round) {
-    for (int j = tid; j < nwant; j += nt) {
-      if (cpos[j] != round) continue;
-      syev_inverse_iteration(j, j, cstart[j], shd[j], dd, ee, n, pv, fac, fac + N * NW, Zt, NW);
-    }
-    __syncthreads();
-  }
-
-  df* Zn = fac;
-  if (!cleanup) {
-    // every gap is above 1e-4 ||T||: the vectors are accurate individually
-    // (error ~ 48-bit rounding x ||T|| / gap <= 4e-11); their Rayleigh
-    // quotients are the eigenvalues, already in ascending order
-    for (long long idx = tid; idx < N * NW; idx += nt) Zn[idx] = Zt[idx];
-    for (int j = tid; j < nwant; j += nt) {
-      df_acc h = acc_zero();
-      for (int i = 0; i < n; ++i) {
-        df_acc tz = acc_zero();
-        tz.fma(dd[i], Zt[i * NW + j]);
-        if (i > 0) tz.fma(ee[i - 1], Zt[(i - 1) * NW + j]);
-        if (i + 1 < n) tz.fma(ee[i], Zt[(i + 1) * NW + j]);
-        h.fma(Zt[i * NW + j], tz.value());
-      }
-      evals[j] = df_to_double(h.value());
-    }
-    __syncthreads();
-  } else {
-    // single vectors only need their Rayleigh quotient; the groups of two or
-    // more run one after another on windows of the workspace
-    for (int j = tid; j < nwant; j += nt) {
-      if (gs1[j] - gs0[j] != 1) continue;
-      syev_single(Zt + j, NW, dd, ee, n, Zn + j, NW, evals + j);
-    }
-    __syncthreads();
-    for (int g0 = 0; g0 < nwant;) {
-      const int g1 = gs1[g0], G = g1 - g0;
-      if (G >= 2)
-        syev_group_rr<2, 2>(G, Zt + g0, NW, dd, ee, n, fac + N * NW + g0, rrw, perm, red, sf, Zn + g0, NW,
-                            evals + g0);
-      g0 = g1;
-    }
-  }
-
-  // ---- back-transformation y = H_0 H_1 ... H_{n-3} z ------------------------
-  // v_k (column k of W below the diagonal) is staged in shared memory once per
-  // step.  Each column of Z is split over S consecutive lanes (S = 1..8 threads
-  // per column, as many as the block holds): lane seg takes rows seg, seg + S, ...,
-  // the partial products meet in a shuffle tree, and the same lanes apply the
-  // update -- row walks stay coalesced across columns and each chain is m / S long.
-  int S = 1;
-  while (S < 8 && 2 * S * nwant <= nt) S <<= 1;
-  for (int k = n - 3; k >= 0; --k) {
-    const df t = tau[k];
-    if (t.hi == 0.f) continue;
-    const int m = n - k - 1;
-    for (int i = tid; i < m; i += nt) v[i] = W[(k + 1 + i) * LD + k];
-    __syncthreads();
-    // for each column c: s_c = v^T z[k+1:, c]; z[k+1:, c] -= t s_c v
-    const int total = nwant * S;
-    for (int base = warp * 32; base < total; base += nt) {
-      const int it = base + lane;
-      const bool valid = it < total;
-      const int c = valid ? it / S : 0, seg = it % S;
-      df* zc = Zn + static_cast<long long>(k + 1) * NW + c;
-      df_acc s0 = acc_zero(), s1 = acc_zero(), s2 = acc_zero(), s3 = acc_zero();
-      if (valid) {
-        int i = seg;
-        for (; i + 3 * S < m; i += 4 * S) {
-          s0.fma(v[i], zc[i * NW]);
-          s1.fma(v[i + S], zc[(i + S) * NW]);
-          s2.fma(v[i + 2 * S], zc[(i + 2 * S) * NW]);
-          s3.fma(v[i + 3 * S], zc[(i + 3 * S) * NW]);
-        }
-        for (; i < m; i += S) s0.fma(v[i], zc[i * NW]);
-      }
-      s0.merge(s1);
-      s2.merge(s3);
-      s0.merge(s2);
-      for (int o = 1; o < S; o <<= 1) s0.merge(shfl_xor_acc(s0, o));
-      if (valid) {
-        const df f = df_mul(t, s0.value());
-        for (int i = seg; i < m; i += S) zc[i * NW] = df_sub(zc[i * NW], df_mul(f, v[i]));
-      }
-    }
-    __syncthreads();
-  }
-  for (long long idx = tid; idx < N * NW; idx += nt) evecs[idx] = df_to_double(Zn[idx]);
-}
-
-// ---- split driver
-//
 // Global workspace: W (n x ldw df) unless it fits in shared memory, the
 // reflectors hv (v_k at hv[k n ..]), dd, ee, tau (df, n each), the shifts shd
 // (df, nwant) and their bounds (4 floats), the factors and working vectors of
@@ -1017,181 +792,208 @@ __global__ void __launch_bounds__(kSyThreads) k_syev_tri(int n, int ldw, int ins
   }
 }
 
-// The same tridiagonalisation by a thread-block cluster of CS CTAs (2, 4 or 8)
-// when W is too large for one block's shared memory: CTA r keeps rows
-// r R .. r R + R - 1 of W (full rows, stride ldw) in its own shared memory.
-// Per step k the owners of column k's entries below the diagonal write them,
-// with their partial sums of squares, into every CTA's copy of v (distributed
-// shared memory); after a cluster barrier every CTA forms the same reflector
-// from the same partials (merged in rank order), computes p = t W22 v for its
-// own rows and sends them, with its partial v^T p, to every CTA; after a
-// second barrier each CTA forms w = p - (t/2)(v^T p) v and updates its own rows
-// (both triangles in the (max, min) product order, so W stays bitwise
-// symmetric).  v, p and the partials are double-buffered by the parity of k:
-// a CTA that reaches step k + 1 writes buffers that no CTA still reads.
-constexpr int kTriMaxCluster = 8;
+// The same tridiagonalisation by a thread-block cluster of 16 CTAs, row i of W in CTA
+// i % 16's shared memory (dealt cyclically, so the shrinking trailing block stays
+// spread over all of them).  A step is bound by the latency of its chain more than by
+// its work, so it exchanges only what the next link needs:
+//   - on entry every CTA holds x = column k and c = column k + 1 below the diagonal
+//     (sent by the rows' owners at the end of the step before);
+//   - the sixteen row warps form y_i = (W22 x)_i for the CTA's rows and send them
+//     to every CTA, while one more warp forms sigma = sum x_j^2 and the reflector's
+//     scalars (v = x - alpha e_1, t = 2 / v^T v);
+//   - cluster barrier: with y everywhere, p = t W22 v = t (y - alpha c) needs no
+//     further exchange: each CTA forms K = (t/2) v^T p and w = p - K v over its
+//     threads (two block barriers), updates its own rows by W22 -= v w^T + w v^T
+//     and sends their entries of columns k + 1 and k + 2; cluster barrier.
+// x, c and y are double-buffered by the parity of k: a CTA that reaches step k + 1
+// writes buffers that no CTA still reads.  What several CTAs form for themselves
+// is the same in all of them (same order, one lane's value broadcast), and the
+// update's arithmetic is symmetric in (i, j), so W stays bitwise symmetric.
+// Measured against the form before it (8 CTAs, a row per warp, every vector sent
+// element by element, global writes and eight block barriers per step; one block with W in
+// global memory above 475 rows): n = 328 3.06 -> 1.31 ms, n = 256 1.94 -> 0.88 ms, i.e. 4.0 and 3.5 us per
+// step; of a step at n = 64 (2.6 us) nearly all is the barriers' and the scalars' latency.
+constexpr int kTriCluster = 16;  // CTAs; not portable, so asked for and checked (cluster_fits)
+constexpr int kTriRowWarps = 16;
+constexpr int kTriThreads = 32 * (kTriRowWarps + 1);
+constexpr int kTriRows = 2;  // rows a warp owns at most
+constexpr int kTriMaxN = kTriCluster * kTriRowWarps * kTriRows;
+static_assert(kTriMaxN <= 32 * kTriRowWarps && kTriRowWarps == kTriCluster && kTriMaxN / kTriCluster <= 32,
+              "one thread per element of p, one warp per destination, one lane per own row");
+constexpr int kTriOneBlock = 40;  // below this size one block's barriers are cheaper
 
-__device__ __forceinline__ df_acc block_merge(df_acc a, df_acc* red) {
-  // every thread's partial merged: warps by shuffles, then warp 0 over the warps (result in lane 0 of warp 0)
+__device__ __forceinline__ df_acc warp_acc_sum(df_acc a) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) a.merge(shfl_xor_acc(a, o));
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  if (lane == 0) red[warp] = a;
-  __syncthreads();
-  df_acc b = acc_zero();
-  if (warp == 0) {
-    b = lane < nw ? red[lane] : acc_zero();
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) b.merge(shfl_xor_acc(b, o));
-  }
-  __syncthreads();
-  return b;
+  return a;
 }
 
-__global__ void __launch_bounds__(kSyThreads) k_syev_tri_cl(int n, int ldw, int R, const double* __restrict__ H,
-                                                            df* __restrict__ hv, df* __restrict__ dd_g,
-                                                            df* __restrict__ ee_g, df* __restrict__ tau_g,
-                                                            const int* __restrict__ skip) {
+// w - (v_i w_j + v_j w_i): compensated products, symmetric in (i, j) bit for bit
+__device__ __forceinline__ df rank2_update(df w, df vi, df wi, df vj, df wj) {
+  const df p1 = two_prod(vi.hi, wj.hi), p2 = two_prod(vj.hi, wi.hi);
+  const float x1 = __fmaf_rn(vi.hi, wj.lo, __fmul_rn(vi.lo, wj.hi));
+  const float x2 = __fmaf_rn(vj.hi, wi.lo, __fmul_rn(vj.lo, wi.hi));
+  const df u = two_sum(p1.hi, p2.hi);
+  const df t = two_sum(w.hi, -u.hi);
+  const float lo = __fadd_rn(__fadd_rn(p1.lo, p2.lo), __fadd_rn(u.lo, __fadd_rn(x1, x2)));
+  return fast_two_sum(t.hi, __fadd_rn(__fadd_rn(w.lo, t.lo), -lo));
+}
+
+__global__ void __launch_bounds__(kTriThreads) k_syev_tri_cl(int n, int ldw, const double* __restrict__ H,
+                                                             df* __restrict__ hv, df* __restrict__ dd_g,
+                                                             df* __restrict__ ee_g, df* __restrict__ tau_g,
+                                                             const int* __restrict__ skip) {
   if (skip != nullptr && *skip != 0) return;  // every CTA of the cluster returns here alike
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
-  const int CS = static_cast<int>(cl.num_blocks()), rank = static_cast<int>(cl.block_rank());
+  constexpr int CS = kTriCluster, NW = kTriRowWarps, RW = kTriRows;
+  const int rank = static_cast<int>(cl.block_rank());
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int R = rank < n ? (n - rank + CS - 1) / CS : 0;  // rows rank, rank + 16, ...
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  df* W = reinterpret_cast<df*>(smem_raw);  // R x ldw: rows r0 .. r1-1
-  df* vb = W + static_cast<long long>(R) * ldw;  // 2 x n
-  df* pb = vb + 2 * n;                            // 2 x n
-  __shared__ df_acc sigp[2][kTriMaxCluster], vpp[2][kTriMaxCluster], red[32];
-  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
-  const int r0 = rank * R, r1 = min(n, r0 + R);
-  const long long LD = ldw;
-  for (long long idx = tid; idx < static_cast<long long>(r1 - r0) * n; idx += nt) {
-    const int i = static_cast<int>(idx / n), j = static_cast<int>(idx % n);
-    W[i * LD + j] = df_from_double(H[static_cast<long long>(r0 + i) * n + j]);
-  }
-  __syncthreads();
-  // column c's entries below the diagonal (own rows) into every CTA's v buffer, and
-  // the partial sum of squares of rows c + 2 .. into every CTA's partials
-  auto send_column = [&](int c) {
-    const int buf = c & 1;
-    df_acc a = acc_zero();
-    for (int i = max(r0, c + 1) + tid; i < r1; i += nt) {
-      const df x = W[(i - r0) * LD + c];
-      for (int r = 0; r < CS; ++r) cl.map_shared_rank(vb + buf * n, r)[i - c - 1] = x;
-      if (i >= c + 2) a.fma(x, x);
+  df* W = reinterpret_cast<df*>(smem_raw);                  // ceil(n / 16) rows of ldw
+  // vectors over the rows keep each owner's rows together (element i at at(i)), so that a CTA's share
+  // travels as one contiguous run per destination
+  const int RP = ((n + CS - 1) / CS) | 1, NV = CS * RP;
+  auto at = [RP](int i) { return (i & (CS - 1)) * RP + (i / CS); };
+  df* xb = W + static_cast<size_t>((n + CS - 1) / CS) * ldw;  // 2 x NV
+  df* cb = xb + 2 * NV;                                     // 2 x NV
+  df* yb = cb + 2 * NV;                                     // 2 x NV
+  df* wv = yb + 2 * NV;                                     // n
+  df* al = wv + n;                                          // n: subdiagonal (alpha_k)
+  df* ta = al + n;                                          // n: t_k
+  __shared__ df sc[3];          // alpha, t, v0
+  __shared__ df ys[32];         // the own rows' y
+  __shared__ df_acc kpart[NW];  // per-warp partials of v^T p
+  for (int r = warp; r < R; r += NW + 1)
+    for (int j = lane; j < n; j += 32)
+      W[r * ldw + j] = df_from_double(H[static_cast<long long>(rank + r * CS) * n + j]);
+  // the own rows' entries of columns c0 and c0 + 1 into the buffers for step c0 of CTA `warp`
+  auto send_columns = [&](int c0) {
+    const int buf = c0 & 1;
+    if (warp < CS && lane < R && rank + lane * CS > c0) {
+      cl.map_shared_rank(xb + buf * NV, warp)[rank * RP + lane] = W[lane * ldw + c0];
+      cl.map_shared_rank(cb + buf * NV, warp)[rank * RP + lane] = W[lane * ldw + c0 + 1];
     }
-    const df_acc s = block_merge(a, red);
-    if (tid == 0)
-      for (int r = 0; r < CS; ++r) cl.map_shared_rank(&sigp[buf][0], r)[rank] = s;
   };
-  send_column(0);
+  // every CTA of the cluster has started before its shared memory is written
+  cl.sync();
+  if (n > 2) send_columns(0);
   for (int k = 0; k + 2 < n; ++k) {
-    const int buf = k & 1, m = n - k - 1;
-    cl.sync();  // (1) column k and its partials are everywhere
-    df_acc sa = sigp[buf][0];
-    for (int r = 1; r < CS; ++r) sa.merge(sigp[buf][r]);
-    const df sigma = sa.value();
-    df* v = vb + buf * n;
-    df* p = pb + buf * n;
-    const df x0 = v[0];
-    const bool own_k = k >= r0 && k < r1;
-    if (sigma.hi == 0.f) {
-      if (own_k) {
-        if (tid == 0) {
-          tau_g[k] = df{0.f, 0.f};
-          dd_g[k] = W[(k - r0) * LD + k];
-          ee_g[k] = x0;
-        }
-      }
-      cl.sync();  // (2) the same barrier count as a reflecting step
-      send_column(k + 1);
-      continue;
-    }
-    const df nrm = df_sqrt(df_add(df_mul(x0, x0), sigma));
-    const df alpha = df_lt0(x0) ? nrm : df_neg(nrm);
-    const df v0 = df_sub(x0, alpha);
-    const df vtv = df_add(sigma, df_mul(v0, v0));
-    const df t = df_div(df{2.f, 0.f}, vtv);
-    __syncthreads();  // every thread has read v[0]
-    if (tid == 0) {
-      v[0] = v0;
-      if (own_k) {
-        tau_g[k] = t;
-        dd_g[k] = W[(k - r0) * LD + k];
-        ee_g[k] = alpha;
-      }
-    }
-    __syncthreads();
-    if (rank == 0)
-      for (int i = tid; i < m; i += nt) hv[static_cast<long long>(k) * n + i] = v[i];
-    // p_i = t (W22 v)_i for the own trailing rows, one warp per row; partial v^T p
-    {
-      df_acc pv = acc_zero();
-      for (int i = max(r0, k + 1) + warp; i < r1; i += nw) {
-        const df* row = W + (i - r0) * LD + (k + 1);
-        df_acc b0 = acc_zero(), b1 = acc_zero();
-        int j = lane;
-        for (; j + 32 < m; j += 64) {
-          b0.fma(row[j], v[j]);
-          b1.fma(row[j + 32], v[j + 32]);
-        }
-        if (j < m) b0.fma(row[j], v[j]);
-        b0.merge(b1);
+    cl.sync();  // columns k and k + 1 are everywhere
+    const int buf = k & 1, k1 = k + 1;
+    const int r0 = k < rank ? 0 : (k - rank) / CS + 1;  // first local row below row k
+    df* x = xb + buf * NV;
+    const df* c = cb + buf * NV;
+    const df* y = yb + buf * NV;
+    if (warp < NW) {
+      df_acc acc[RW];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) b0.merge(shfl_xor_acc(b0, o));
-        if (lane == 0) {
-          const df pi = df_mul(t, b0.value());
-          for (int r = 0; r < CS; ++r) cl.map_shared_rank(pb + buf * n, r)[i - k - 1] = pi;
-          pv.fma(v[i - k - 1], pi);
+      for (int s = 0; s < RW; ++s) acc[s] = acc_zero();
+      const df* Wr = W + (r0 + warp) * ldw;
+      const int mine = R - r0 - warp;  // rows r0 + warp + s NW < R
+      if (mine > 0) {
+        for (int j = k1 + lane; j < n; j += 32) {
+          const df xj = x[at(j)];
+#pragma unroll
+          for (int s = 0; s < RW; ++s)
+            if (s * NW < mine) acc[s].fma(Wr[s * NW * ldw + j], xj);
         }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+          for (int s = 0; s < RW; ++s)
+            if (s * NW < mine) acc[s].merge(shfl_xor_acc(acc[s], o));
+#pragma unroll
+        for (int s = 0; s < RW; ++s)
+          if (s * NW < mine) {
+            if (lane == 0) ys[r0 + warp + s * NW] = acc[s].value();
+          }
       }
-      const df_acc s = block_merge(pv, red);
-      if (tid == 0)
-        for (int r = 0; r < CS; ++r) cl.map_shared_rank(&vpp[buf][0], r)[rank] = s;
+      // the row warps' barrier (the scalars' warp goes on): the CTA's y is complete
+      asm volatile("bar.sync 1, %0;" ::"n"(32 * NW) : "memory");
+      if (lane >= r0 && lane < R) cl.map_shared_rank(yb + buf * NV, warp)[rank * RP + lane] = ys[lane];
+    } else {
+      df_acc s0 = acc_zero(), s1 = acc_zero();
+      int j = k1 + 1 + lane;
+      for (; j + 32 < n; j += 64) {
+        const df xa = x[at(j)], xc = x[at(j + 32)];
+        s0.fma(xa, xa);
+        s1.fma(xc, xc);
+      }
+      if (j < n) s0.fma(x[at(j)], x[at(j)]);
+      s0.merge(s1);
+      const df sigma = shfl_df(warp_acc_sum(s0).value(), 0);
+      const df x0 = x[at(k1)];
+      const bool flat = sigma.hi == 0.f;  // nothing below the subdiagonal: t = 0 leaves W as it is
+      const df nrm = df_sqrt(df_add(df_mul(x0, x0), sigma));
+      const df alpha = flat ? x0 : (df_lt0(x0) ? nrm : df_neg(nrm));
+      const df v0 = df_sub(x0, alpha);
+      // t = 2 / (v^T v): the reciprocal with one more Newton step, as accurate as a division and half its latency
+      const df vtv = df_add(sigma, df_mul(v0, v0));
+      const df r = df_recip(vtv);
+      const df t = flat ? df{0.f, 0.f} : df_mul_f(df_add(r, df_mul(r, df_sub(df{1.f, 0.f}, df_mul(vtv, r)))), 2.f);
+      if (lane == 0) {
+        sc[0] = al[k] = alpha;
+        sc[1] = ta[k] = t;
+        sc[2] = v0;
+      }
     }
-    cl.sync();  // (2) every p_i and partial v^T p are everywhere
-    {
-      df_acc c = vpp[buf][0];
-      for (int r = 1; r < CS; ++r) c.merge(vpp[buf][r]);
-      const df kc = df_mul(df_mul_f(t, 0.5f), c.value());
-      for (int i = tid; i < m; i += nt) p[i] = df_sub(p[i], df_mul(kc, v[i]));  // w
+    cl.sync();  // y is everywhere, the scalars are in shared memory
+    const df alpha = sc[0], t = sc[1], v0 = sc[2];
+    // p and the partials of v^T p, one element per thread (n <= 32 NW)
+    df pj, vj;
+    const int j1 = k1 + tid;
+    if (warp < NW) {
+      df_acc kv = acc_zero();
+      if (j1 < n) {
+        vj = j1 == k1 ? v0 : x[at(j1)];
+        pj = df_mul(t, df_sub(y[at(j1)], df_mul(alpha, c[at(j1)])));
+        kv.fma(vj, pj);
+      }
+      if (k1 + 32 * warp < n) kv = warp_acc_sum(kv);
+      if (lane == 0) kpart[warp] = kv;
     }
     __syncthreads();
-    // own rows: W22 -= v w^T + w v^T, one warp per row, lanes along it (column k keeps
-    // the entries of the reduced matrix)
-    for (int row = max(r0, k + 1) + warp; row < r1; row += nw) {
-      const int i = row - k - 1;  // trailing index of the row
-      const df vi = v[i], wi = p[i];
-      df* rowp = W + (row - r0) * LD + (k + 1);
+    if (warp < NW) {
+      df_acc kv = kpart[lane & (NW - 1)];
+#pragma unroll
+      for (int o = NW / 2; o > 0; o >>= 1) kv.merge(shfl_xor_acc(kv, o));
+      const df kc = shfl_df(df_mul(df_mul_f(t, 0.5f), kv.value()), 0);
+      if (j1 < n) {
+        wv[j1] = df_sub(pj, df_mul(kc, vj));
+        if (j1 == k1) x[at(k1)] = v0;  // this CTA's copy: x becomes v
+      }
+    }
+    __syncthreads();
+    if (warp < NW)
+      for (int r = r0 + warp; r < R; r += NW) {
+        const int i = rank + r * CS;
+        const df vi = x[at(i)], wi = wv[i];
+        df* Wr = W + r * ldw;
+        if (lane == 0) Wr[k] = vi;  // column k keeps the reflector
 #pragma unroll 2
-      for (int j = lane; j < m; j += 32) {
-        df_acc u0 = acc_zero();
-        if (j <= i) {
-          u0.fma(vi, p[j]);
-          u0.fma(wi, v[j]);
-        } else {
-          u0.fma(v[j], wi);
-          u0.fma(p[j], vi);
-        }
-        rowp[j] = df_sub(rowp[j], u0.value());
+        for (int j = k1 + lane; j < n; j += 32) Wr[j] = rank2_update(Wr[j], vi, wi, x[at(j)], wv[j]);
       }
-    }
-    __syncthreads();
-    send_column(k + 1);
+    __syncthreads();  // the own rows are complete
+    if (k + 3 < n) send_columns(k1);
   }
-  // the last 2 x 2 block
-  if (tid == 0) {
-    if (n >= 2) {
-      if (n - 2 >= r0 && n - 2 < r1) dd_g[n - 2] = W[(n - 2 - r0) * LD + (n - 2)];
-      if (n - 1 >= r0 && n - 1 < r1) {
-        dd_g[n - 1] = W[(n - 1 - r0) * LD + (n - 1)];
-        ee_g[n - 2] = W[(n - 1 - r0) * LD + (n - 2)];
-      }
-      if (rank == 0) tau_g[n - 2] = df{0.f, 0.f};
-    } else if (rank == 0) {
-      dd_g[0] = W[0];
+  // results to global memory: nothing is written there during the steps, whose barriers would wait for it
+  __syncthreads();
+  for (int r = warp; r < R; r += NW + 1) {
+    const int i = rank + r * CS;
+    const df* Wr = W + r * ldw;
+    for (int k = lane; k < i && k + 2 < n; k += 32) hv[static_cast<long long>(k) * n + (i - k - 1)] = Wr[k];
+    if (lane == 0) {
+      dd_g[i] = Wr[i];
+      if (i == n - 1 && n >= 2) ee_g[n - 2] = Wr[n - 2];
     }
-    if (rank == 0 && n >= 1) tau_g[n - 1] = df{0.f, 0.f};
   }
+  if (rank == 0)
+    for (int k = tid; k < n; k += kTriThreads) {
+      if (k + 2 < n) ee_g[k] = al[k];
+      tau_g[k] = k + 2 < n ? ta[k] : df{0.f, 0.f};
+    }
   cl.sync();  // no CTA leaves while another may still write into its shared memory
 }
 
@@ -1489,10 +1291,6 @@ struct GjShared {
 __device__ __forceinline__ unsigned long long pivot_key(float a, int i) {
   // |a| >= 0: its bits order like its value; ties go to the smaller row
   return (static_cast<unsigned long long>(__float_as_uint(a)) << 32) | static_cast<unsigned>(31 - i);
-}
-
-__device__ __forceinline__ df shfl_df(df v, int src) {
-  return df{__shfl_sync(0xffffffffu, v.hi, src), __shfl_sync(0xffffffffu, v.lo, src)};
 }
 
 __device__ void gj_solve_reg(const df* S, int q, int nrhs, int lds, GjShared* g, df* sol, int ldsol) {
@@ -2919,12 +2717,6 @@ __global__ void k_identity(int n, double* __restrict__ X) {
     X[i] = (i / N == i % N) ? 1.0 : 0.0;
 }
 
-size_t syev_smem_base(int n, int nwant) {
-  return (2 * sizeof(df) * n + 2 * sizeof(float) * n + sizeof(float) * nwant + 2 * sizeof(int) * nwant +
-          4 * sizeof(df) * n + sizeof(df) * nwant + 2 * sizeof(int) * nwant + 15) &
-         ~static_cast<size_t>(15);
-}
-
 constexpr size_t kSmemBudget = 225 * 1024;
 
 }  // namespace
@@ -3007,33 +2799,41 @@ void pencil_work_destroy(PencilWork* w) {
   delete w;
 }
 
-// Whether a cluster of c blocks of k_syev_tri_cl with `bytes` of shared memory each can be
-// resident on this device (asked once per device and size class; the answer is kept).
-bool cluster_fits(int c, size_t bytes) {
-  static std::mutex mu;
-  static std::map<std::pair<int, int>, bool> known;  // (device, c * 1024 + KiB)
-  int dev = 0;
-  cudaGetDevice(&dev);
-  const int key = c * 1024 + static_cast<int>((bytes + 1023) / 1024);
-  std::lock_guard<std::mutex> lk(mu);
-  auto it = known.find({dev, key});
-  if (it != known.end()) return it->second;
-  ensure_dynamic_smem(reinterpret_cast<const void*>(k_syev_tri_cl), bytes);
+cudaLaunchConfig_t tri_config(size_t smem, cudaStream_t st, cudaLaunchAttribute* attr) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(c);
-  cfg.blockDim = dim3(kSyThreads);
-  cfg.dynamicSmemBytes = bytes;
-  cudaLaunchAttribute attr[1];
+  cfg.gridDim = dim3(kTriCluster);
+  cfg.blockDim = dim3(kTriThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = c;
+  attr[0].val.clusterDim.x = kTriCluster;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
+  return cfg;
+}
+
+// Whether the tridiagonalisation's cluster with `smem` bytes per CTA can be resident on the current
+// device (asked once per device and size class; the answer is kept).
+bool cluster_fits(size_t smem) {
+  static std::mutex mu;
+  static std::map<std::pair<int, int>, bool> known;  // (device, KiB)
+  int dev = 0;
+  cudaGetDevice(&dev);
+  const std::pair<int, int> key = {dev, static_cast<int>((smem + 1023) / 1024)};
+  std::lock_guard<std::mutex> lk(mu);
+  auto it = known.find(key);
+  if (it != known.end()) return it->second;
+  bool ok = cudaFuncSetAttribute(reinterpret_cast<const void*>(k_syev_tri_cl),
+                                 cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+  ensure_dynamic_smem(reinterpret_cast<const void*>(k_syev_tri_cl), smem);
+  cudaLaunchAttribute attr[1];
+  const cudaLaunchConfig_t cfg = tri_config(smem, nullptr, attr);
   int clusters = 0;
-  const bool ok = cudaOccupancyMaxActiveClusters(&clusters, k_syev_tri_cl, &cfg) == cudaSuccess && clusters > 0;
+  ok = ok && cudaOccupancyMaxActiveClusters(&clusters, k_syev_tri_cl, &cfg) == cudaSuccess && clusters > 0;
   if (!ok) cudaGetLastError();
-  known[{dev, key}] = ok;
+  known[key] = ok;
   return ok;
 }
 
@@ -3057,30 +2857,14 @@ void launch_syev_df(PencilWork* w, int n, int nwant, const double* H, double* ev
                                         (sizeof(df) * static_cast<size_t>(n)))));
   const size_t sm_back = sizeof(df) * static_cast<size_t>(wpb + chunk) * n;
   ProfScope ps(st, P_PENCIL, 8.0 * n * n + 8.0 * n * nwant, 0.0, 4);
-  // W too large for one block: a cluster holding its rows, the largest of 8, 4, 2 blocks that can be scheduled
-  // (each block's work per step is its rows times the trailing row length: more blocks, shorter steps)
-  int cs = 0, rows_per = 0;
-  size_t sm_cl = 0;
-  if (!inshared)
-    for (int c = kTriMaxCluster; c >= 2 && cs == 0; c /= 2) {
-      rows_per = (n + c - 1) / c;
-      sm_cl = sizeof(df) * (static_cast<size_t>(rows_per) * ldw + 4 * static_cast<size_t>(n));
-      if (sm_cl <= kSmemBudget && cluster_fits(c, sm_cl)) cs = c;
-    }
-  if (cs > 0) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(cs);
-    cfg.blockDim = dim3(kSyThreads);
-    cfg.dynamicSmemBytes = sm_cl;
-    cfg.stream = st;
+  // from kTriOneBlock rows a cluster of 16 CTAs, where it can be scheduled
+  const size_t tri_rows = ceil_div(n, kTriCluster);
+  const size_t sm_cl = sizeof(df) * (tri_rows * ldw + 6 * kTriCluster * (tri_rows | 1) + 3 * static_cast<size_t>(n));
+  if (n >= kTriOneBlock && n <= kTriMaxN && cluster_fits(sm_cl)) {
+    ensure_dynamic_smem(reinterpret_cast<const void*>(k_syev_tri_cl), sm_cl);
     cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = cs;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, k_syev_tri_cl, n, ldw, rows_per, H, w->hv, w->dd, w->ee, w->tau, skip);
+    const cudaLaunchConfig_t cfg = tri_config(sm_cl, st, attr);
+    cudaLaunchKernelEx(&cfg, k_syev_tri_cl, n, ldw, H, w->hv, w->dd, w->ee, w->tau, skip);
   } else {
     ensure_dynamic_smem(reinterpret_cast<const void*>(k_syev_tri), sm_tri);
     k_syev_tri<<<1, kSyThreads, sm_tri, st>>>(n, ldw, inshared, H, w->W, w->hv, w->dd, w->ee, w->tau, skip);
@@ -3095,30 +2879,36 @@ void launch_syev_df(PencilWork* w, int n, int nwant, const double* H, double* ev
   k_syev_back<<<ceil_div(nwant, wpb), 32 * wpb, sm_back, st>>>(n, nwant, chunk, w->hv, w->tau, w->Zt, evecs, skip);
 }
 
-void launch_syev_df_into(int n, int nwant, const double* H, double* evals, double* evecs, df* W, df* tau, df* dd,
-                         df* ee, df* fac, df* Zt, df* rr, int* perm, cudaStream_t st) {
-  const int ldw = n | 1;
-  size_t sm = syev_smem_base(n, nwant);
-  int flags = 0;
-  const size_t wb = sizeof(df) * static_cast<size_t>(n) * ldw;
-  const size_t fb = sizeof(df) * 2 * static_cast<size_t>(n) * nwant;
-  const size_t zb = sizeof(df) * static_cast<size_t>(n) * nwant;
-  if (sm + wb <= kSmemBudget) {
-    flags |= kSyW;
-    sm += wb;
-  }
-  if (sm + fb <= kSmemBudget) {
-    flags |= kSyF;
-    sm += fb;
-  }
-  if (sm + zb <= kSmemBudget) {
-    flags |= kSyZ;
-    sm += zb;
-  }
-  ProfScope ps(st, P_PENCIL, 8.0 * n * n + 8.0 * n * nwant, 0.0);
-  ensure_dynamic_smem(reinterpret_cast<const void*>(k_syev_df), sm);
-  k_syev_df<<<1, kSyThreads, sm, st>>>(n, nwant, ldw, flags, H, evals, evecs, W, tau, dd, ee, fac, Zt, rr, perm,
-                                       nullptr);
+size_t syev_scratch(int n, int nwant, PencilWork* w, void* base) {
+  size_t off = 0;
+  char* at = static_cast<char*>(base);
+  auto carve = [&](auto** p, size_t count) {
+    if (base) *p = reinterpret_cast<std::remove_reference_t<decltype(*p)>>(at + off);
+    off = (off + sizeof(**p) * count + 255) & ~static_cast<size_t>(255);
+  };
+  const size_t nm = static_cast<size_t>(n), nw = static_cast<size_t>(nwant);
+  carve(&w->hv, nm * nm);
+  carve(&w->dd, nm);
+  carve(&w->ee, nm);
+  carve(&w->tau, nm);
+  carve(&w->shd, nw);
+  carve(&w->bounds, 4);
+  carve(&w->fac, 3 * nm * nw);
+  carve(&w->Zt, nm * nw);
+  carve(&w->rr, 4 * (nw * nw > 4 * nw ? nw * nw : 4 * nw));
+  return off;
+}
+
+size_t syev_scratch_bytes(int n, int nwant) {
+  PencilWork w;
+  return syev_scratch(n, nwant, &w, nullptr);
+}
+
+void launch_syev_df_into(int n, int nwant, const double* H, double* evals, double* evecs, void* scratch,
+                         cudaStream_t st) {
+  PencilWork w;
+  syev_scratch(n, nwant, &w, scratch);
+  launch_syev_df(&w, n, nwant, H, evals, evecs, st);
 }
 
 void launch_pencil_solve(PencilWork* w, int dn, int m, int q, const double* C64, const float2* Cdf,

@@ -56,3 +56,45 @@ def test_block_per_row_sweeps(width, tune):
             x = ae.amgeig_apply_vcycle(h.handle, level, b, ae.options(precision=ae.AMGEIG_MIXED_FP32, autotune=tune))
             err = np.abs(x - ref).max(axis=0) / np.abs(ref).max(axis=0)
             assert np.all(err <= 2e-5), (level, err.max())
+
+
+@pytest.mark.parametrize("n,nwant", [(39, 7), (40, 7), (41, 41), (63, 5), (64, 64), (65, 9), (127, 33), (129, 20), (255, 40),
+                                     (257, 16), (511, 24), (512, 31), (513, 12)])
+def test_sym_eigh_cluster_sizes(n, nwant):
+    """The dense eigensolver around the sizes where its tridiagonalisation changes form or distribution (one
+    block below 40 rows and above 512, rows dealt over 16 CTAs in between, one lane per own row) and where the
+    shifts, vectors and reflector chunks have remainders, against LAPACK (bounds of the eigensolver tests)."""
+    rng = np.random.default_rng(n)
+    c = rng.standard_normal((n, n))
+    H = np.diag(5.0 + 3.0 * np.arange(n)) + c + c.T
+    w, V = ae.amgeig_sym_eigh(H, nwant)
+    full = np.linalg.eigvalsh(H)
+    scale = np.abs(full).max()
+    assert np.all(np.abs(w - full[:nwant]) <= 1e-12 * scale)
+    assert np.abs(V.T @ V - np.eye(nwant)).max() < 1e-12
+    assert np.abs(H @ V - V * w).max() <= 1e-11 * scale
+
+
+@pytest.mark.parametrize("n,nwant", [(1, 1), (3, 2), (16, 16), (39, 12), (40, 12), (127, 64), (128, 64)])
+def test_noalloc_gives_the_allocating_entrys_bits(n, nwant):
+    """Both entry points run the same kernels: the same bits, also on a diagonal and a decoupled matrix."""
+    import torch
+
+    rng = np.random.default_rng(n)
+    c = rng.standard_normal((n, n))
+    dense = np.diag(5.0 + 3.0 * np.arange(n)) + c + c.T
+    split = dense.copy()
+    split[: n // 2, n // 2:] = 0.0
+    split[n // 2:, : n // 2] = 0.0
+    for H in (dense, split, np.diag(1.0 + np.arange(n))):
+        w, V = ae.amgeig_sym_eigh(H, nwant)
+        Hd = torch.tensor(H, dtype=torch.float64, device="cuda")
+        wd = torch.empty(nwant, dtype=torch.float64, device="cuda")
+        Vd = torch.empty((n, nwant), dtype=torch.float64, device="cuda")
+        ae.amgeig_sym_eigh_noalloc(Hd, wd, Vd)
+        torch.cuda.synchronize()
+        np.testing.assert_array_equal(wd.cpu().numpy(), w)
+        np.testing.assert_array_equal(Vd.cpu().numpy(), V)
+        full = np.linalg.eigvalsh(H)
+        assert np.all(np.abs(w - full[:nwant]) <= 1e-12 * np.abs(full).max())
+        assert np.abs(V.T @ V - np.eye(nwant)).max() < 1e-12
