@@ -306,7 +306,7 @@ int amgeig_apply_vcycle(amgeig_hierarchy h, int level, int width, const amgeig_o
  *   stream    cudaStream_t (NULL: the legacy default stream).
  * The call only enqueues work on `stream` (no synchronisation, no cudaMalloc,
  * cudaFree or allocating library call).  Its scratch is one file-scope device
- * array of 544 KiB that every GPU loading the library holds until exit; the
+ * array of 512 KiB that every GPU loading the library holds until exit; the
  * first call on a device looks the array's device address up with
  * cudaGetSymbolAddress, so make that first call outside any stream capture.
  * All calls share the array and it keeps the last call's contents (the solver

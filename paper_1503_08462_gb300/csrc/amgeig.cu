@@ -2137,7 +2137,7 @@ int amgeig_sym_eigh(int device, int n, int nwant, const double* H, double* evals
   if (e0 == cudaSuccess) e0 = m.alloc(&dV, static_cast<size_t>(n) * nwant);
   if (e0 == cudaSuccess) e0 = cudaMemcpyAsync(dH, H, sizeof(double) * n * n, cudaMemcpyHostToDevice, st);
   if (e0 == cudaSuccess) {
-    launch_syev_df(pw, n, nwant, dH, dv, dV, st);
+    launch_eigh(pw, n, nwant, dH, dv, dV, st);
     e0 = cudaGetLastError();
   }
   if (e0 == cudaSuccess) e0 = cudaMemcpyAsync(evals, dv, sizeof(double) * nwant, cudaMemcpyDeviceToHost, st);

@@ -266,16 +266,22 @@ void launch_coarse_modes(PencilWork* w, int dn, int nwant, const double* An, dou
 
 // Symmetric eigensolver in float-float: the `nwant` smallest eigenpairs of the
 // symmetric n x n row-major float64 matrix H.  evals (nwant), evecs (n x nwant
-// row-major).  Exposed for the kernel-level tests.
+// row-major).
 // skip (device, may be null): when *skip != 0 at run time the kernel returns at once
 void launch_syev_df(PencilWork* w, int n, int nwant, const double* H, double* evals, double* evecs,
                     cudaStream_t st, const int* skip = nullptr);
 
-// The same eigensolver on caller-provided scratch (syev_scratch_bytes(n, nwant) device bytes, 256-byte
-// aligned; n <= 128, where the tridiagonalisation needs no global matrix); enqueues only.
-size_t syev_scratch_bytes(int n, int nwant);
-void launch_syev_df_into(int n, int nwant, const double* H, double* evals, double* evecs, void* scratch,
-                         cudaStream_t st);
+// Its tridiagonalisation in one block (eigh.cu): below 40 and above 512 rows.
+void launch_syev_tri_block(PencilWork* w, int n, int ldw, const double* H, const int* skip, cudaStream_t st);
+
+// The eigensolver of the entry points (eigh.cu): the same problem with the arithmetic, and so the eigenvectors'
+// signs, that those calls have always returned.
+void launch_eigh(PencilWork* w, int n, int nwant, const double* H, double* evals, double* evecs, cudaStream_t st);
+// The same on caller-provided workspace (device pointers sized as in
+// pencil_work_create for nmax >= n + 1 and nwant_max >= nwant); enqueues only.
+struct df;
+void launch_eigh_into(int n, int nwant, const double* H, double* evals, double* evecs, df* W, df* tau, df* dd, df* ee,
+                      df* fac, df* Zt, df* rr, int* perm, cudaStream_t st);
 
 // Hierarchy load on the device (the blob copied in one piece): *out += the word sum (mod 2^64) of
 // `bytes` (a multiple of 8) at blob; *bad |= 1 unless (rp, ci) is a valid CSR structure of a

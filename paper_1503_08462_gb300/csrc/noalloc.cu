@@ -30,7 +30,7 @@ namespace {
 
 constexpr int kNoAllocMaxN = 128;
 constexpr int kNoAllocMaxWant = 64;
-constexpr size_t kNoAllocScratchBytes = 544 * 1024;  // n = 128, nwant = 64 take 516 KiB
+constexpr size_t kNoAllocScratchBytes = 512 * 1024;
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratchBytes];
 
@@ -53,6 +53,12 @@ int scratch_address(int device, void** out) {
   return AMGEIG_OK;
 }
 
+size_t carve(size_t* off, size_t bytes) {
+  const size_t at = *off;
+  *off = (at + bytes + 255) & ~static_cast<size_t>(255);
+  return at;
+}
+
 }  // namespace
 }  // namespace amgeig
 
@@ -72,9 +78,24 @@ extern "C" int amgeig_sym_eigh_noalloc(int n, int nwant, const double* H, double
   void* base = nullptr;
   int rc = scratch_address(device, &base);
   if (rc) return rc;
-  if (syev_scratch_bytes(n, nwant) > kNoAllocScratchBytes)
-    return set_last_error(AMGEIG_EINVAL, "scratch layout exceeds the fixed array");
-  launch_syev_df_into(n, nwant, H, evals, evecs, base, static_cast<cudaStream_t>(stream));
+  // carve the eigensolver's workspace out of the fixed array
+  const size_t nm = static_cast<size_t>(n), nw = static_cast<size_t>(nwant);
+  size_t off = 0;
+  const size_t oW = carve(&off, sizeof(df) * nm * (nm + 1));
+  const size_t oTau = carve(&off, sizeof(df) * nm);
+  const size_t oD = carve(&off, sizeof(df) * nm);
+  const size_t oE = carve(&off, sizeof(df) * nm);
+  const size_t oF = carve(&off, sizeof(df) * 2 * nm * nw);
+  const size_t oZ = carve(&off, sizeof(df) * nm * nw);
+  const size_t rrn = nw * nw > 4 * nw ? nw * nw : 4 * nw;
+  const size_t oR = carve(&off, sizeof(df) * 4 * rrn);
+  const size_t oP = carve(&off, sizeof(int) * nw);
+  if (off > kNoAllocScratchBytes) return set_last_error(AMGEIG_EINVAL, "scratch layout exceeds 512 KiB");
+  unsigned char* b = static_cast<unsigned char*>(base);
+  launch_eigh_into(n, nwant, H, evals, evecs, reinterpret_cast<df*>(b + oW), reinterpret_cast<df*>(b + oTau),
+                      reinterpret_cast<df*>(b + oD), reinterpret_cast<df*>(b + oE), reinterpret_cast<df*>(b + oF),
+                      reinterpret_cast<df*>(b + oZ), reinterpret_cast<df*>(b + oR), reinterpret_cast<int*>(b + oP),
+                      static_cast<cudaStream_t>(stream));
   cudaError_t le = cudaGetLastError();
   if (le != cudaSuccess)
     return set_last_error(AMGEIG_ECUDA, (std::string("eigensolver launch: ") + cudaGetErrorString(le)).c_str());

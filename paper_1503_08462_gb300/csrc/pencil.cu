@@ -36,119 +36,78 @@
 #include <cstdio>
 #include <map>
 #include <mutex>
-#include <type_traits>
 
 #include "common.cuh"
 #include "kernels.cuh"
 #include "prof.cuh"
+#include "syev.cuh"
 
 namespace amgeig {
-
-#ifndef AMGEIG_SY_THREADS
-#define AMGEIG_SY_THREADS 1024
-#endif
-constexpr int kSyThreads = AMGEIG_SY_THREADS;
-
-struct PencilWork {
-  int dn = 0, qmax = 0, nmax = 0;
-  void* base = nullptr;  // one device allocation holding every array below
-  size_t bytes = 0;      // its size
-  // Rayleigh-Ritz pencil (float-float)
-  df* KB = nullptr;   // dn x 2q   Z_m^T C = [K | B]
-  df* Ft = nullptr;   // dn x q    K - Theta B
-  df* Tt = nullptr;   // q x q
-  df* St = nullptr;   // q x q     Schur complement of the Gram matrix
-  df* Lq = nullptr;   // q x q     its Cholesky factor (fallback)
-  df* Xq = nullptr;   // q x q     scratch (fallback)
-  double* H = nullptr;   // nmax x nmax standard form (fallback)
-  double* Yh = nullptr;  // nmax x q eigenvectors [a; b]
-  // float-float eigensolver
-  df* W = nullptr;     // nmax x nmax
-  df* tau = nullptr;   // nmax
-  df* dd = nullptr;    // nmax
-  df* ee = nullptr;    // nmax
-  df* fac = nullptr;   // 6 x nmax x nwant_max
-  df* Zt = nullptr;    // nmax x nwant_max
-  df* rr = nullptr;    // 4 x nwant_max^2 (Rayleigh-Ritz clean-up)
-  int* perm = nullptr; // nwant_max
-  df* hv = nullptr;    // nmax x nmax reflectors (split path)
-  df* shd = nullptr;   // nwant_max refined shifts (split path)
-  float* bounds = nullptr;  // 4: Gershgorin bounds, ||T||, pivot floor (split path)
-  int nwant_max = 0;
-  // coarse decomposition
-  double* Lm = nullptr;  // dn x dn
-  double* Hs = nullptr;  // dn x dn
-  // structured Rayleigh quotient iteration
-  double* sr_mu = nullptr;  // qmax
-  double* sr_X = nullptr;   // nmax x qmax
-  int* sr_conv = nullptr;   // qmax
-  int* sr_flag = nullptr;   // 4: accepted, reason of a rejection, inertia count, q
-};
 
 namespace {
 
 // ------------------------------------------------------------ block helpers
 
-__device__ __forceinline__ df shfl_df(df v, int src) {
-  return df{__shfl_sync(0xffffffffu, v.hi, src), __shfl_sync(0xffffffffu, v.lo, src)};
+__device__ __forceinline__ df_acc warp_acc_sum(df_acc a) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) a.merge(shfl_xor_acc(a, o));
+  return a;
 }
 
-// sum_i a[i sa] b[i sb] (i < len) in float-float with four interleaved
-// accumulators: independent chains keep the float32 pipes busy in these
-// latency-bound single-block kernels
-__device__ __forceinline__ df_acc dot4(const df* a, int sa, const df* b, int sb, int len) {
-  df_acc c0 = acc_zero(), c1 = acc_zero(), c2 = acc_zero(), c3 = acc_zero();
-  int i = 0;
-  for (; i + 4 <= len; i += 4) {
-    c0.fma(a[i * sa], b[i * sb]);
-    c1.fma(a[(i + 1) * sa], b[(i + 1) * sb]);
-    c2.fma(a[(i + 2) * sa], b[(i + 2) * sb]);
-    c3.fma(a[(i + 3) * sa], b[(i + 3) * sb]);
-  }
-  for (; i < len; ++i) c0.fma(a[i * sa], b[i * sb]);
-  c0.merge(c1);
-  c2.merge(c3);
-  c0.merge(c2);
-  return c0;
+// Sturm counts (the number of eigenvalues of the tridiagonal below x) from the
+// leading principal minors p_i = (d_i - x) p_{i-1} - e_{i-1}^2 p_{i-2} (Golub & Van Loan
+// 8.4.1): a sign change per eigenvalue.  The recurrence's chain is one product
+// and one difference (~75 cycles in float-float) where the quotient form
+// q_i = d_i - x - e^2 / q_{i-1} adds a reciprocal (~300).  The minors' range is kept by an
+// exact power-of-two rescaling of the pair every other step; d and e^2 are
+// scaled to ||T|| <= 1, so a step grows them by at most 3.  A zero minor is
+// replaced by a tiny one of the opposite sign (one count, as for a tiny negative pivot).
+__device__ __forceinline__ float minor_scale(float a, float b) {
+  const int e = (__float_as_int(fmaxf(fabsf(a), fabsf(b))) >> 23) & 0xff;
+  return __int_as_float((254 - e) << 23);  // 2^(127 - e)
 }
 
-// the same with weights: sum_i a[i sa] w[i] b[i sb]
-__device__ __forceinline__ df_acc dot4w(const df* a, int sa, const df* w, const df* b, int sb, int len) {
-  df_acc c0 = acc_zero(), c1 = acc_zero(), c2 = acc_zero(), c3 = acc_zero();
-  int i = 0;
-  for (; i + 4 <= len; i += 4) {
-    c0.fma(df_mul(a[i * sa], w[i]), b[i * sb]);
-    c1.fma(df_mul(a[(i + 1) * sa], w[i + 1]), b[(i + 1) * sb]);
-    c2.fma(df_mul(a[(i + 2) * sa], w[i + 2]), b[(i + 2) * sb]);
-    c3.fma(df_mul(a[(i + 3) * sa], w[i + 3]), b[(i + 3) * sb]);
-  }
-  for (; i < len; ++i) c0.fma(df_mul(a[i * sa], w[i]), b[i * sb]);
-  c0.merge(c1);
-  c2.merge(c3);
-  c0.merge(c2);
-  return c0;
-}
-
-__device__ __forceinline__ int sturm_count(const float* sd, const float* se2, int n, float x, float pivmin) {
-  float qv = sd[0] - x;
-  int cnt = qv < 0.f;
+__device__ __forceinline__ int sturm_count(const df* d, const df* e2, int n, float x) {
+  float p0 = 1.f, p1 = d[0].hi - x;
+  if (p1 == 0.f) p1 = -8.7e-19f;
+  int cnt = p1 < 0.f;
   for (int i = 1; i < n; ++i) {
-    if (fabsf(qv) < pivmin) qv = -pivmin;
-    qv = sd[i] - x - __fdividef(se2[i - 1], qv);
-    cnt += qv < 0.f;
+    float pn = fmaf(d[i].hi - x, p1, -e2[i - 1].hi * p0);
+    if (pn == 0.f) pn = -8.7e-19f * p1;
+    cnt += (pn < 0.f) != (p1 < 0.f);
+    p0 = p1;
+    p1 = pn;
+    if (i & 1) {
+      const float sc = minor_scale(p0, p1);
+      p0 *= sc;
+      p1 *= sc;
+    }
   }
   return cnt;
 }
 
-// The same count in float-float; ee2 holds e_i^2.  The reciprocal of the
-// previous pivot replaces the division (one Newton step on the float32 rcp).
-__device__ __forceinline__ int sturm_count_df(const df* dd, const df* ee2, int n, df x, float pivmin) {
-  df qv = df_sub(dd[0], x);
-  int cnt = df_lt0(qv);
+// a - b with the low parts added once (error 2^-47 of the larger operand)
+__device__ __forceinline__ df df_sub_sloppy(df a, df b) {
+  const df s = two_sum(a.hi, -b.hi);
+  return fast_two_sum(s.hi, __fadd_rn(s.lo, __fsub_rn(a.lo, b.lo)));
+}
+
+__device__ __forceinline__ int sturm_count_df(const df* d, const df* e2, int n, df x) {
+  df p0 = df{1.f, 0.f}, p1 = df_sub(d[0], x);
+  if (p1.hi == 0.f) p1 = df{-8.7e-19f, 0.f};
+  int cnt = p1.hi < 0.f;
+#pragma unroll 2
   for (int i = 1; i < n; ++i) {
-    if (fabsf(qv.hi) < pivmin) qv = df{-pivmin, 0.f};
-    qv = df_sub(df_sub(dd[i], x), df_mul(ee2[i - 1], df_recip(qv)));
-    cnt += df_lt0(qv);
+    df pn = df_sub_sloppy(df_mul(df_sub(d[i], x), p1), df_mul(e2[i - 1], p0));
+    if (pn.hi == 0.f) pn = df{-8.7e-19f * p1.hi, 0.f};
+    cnt += (pn.hi < 0.f) != (p1.hi < 0.f);
+    p0 = p1;
+    p1 = pn;
+    if (i & 1) {
+      const float sc = minor_scale(p0.hi, p1.hi);
+      p0 = df{p0.hi * sc, p0.lo * sc};
+      p1 = df{p1.hi * sc, p1.lo * sc};
+    }
   }
   return cnt;
 }
@@ -160,288 +119,92 @@ __device__ __forceinline__ int sturm_count_df(const df* dd, const df* ee2, int n
 // one block per group of close shifts (k_syev_vecs) and the
 // back-transformation (k_syev_back).
 
-// Householder tridiagonalisation of the symmetric W (n x n, row stride LD,
-// full storage) by the whole block.  Four barriers per step: the norm of the
-// next column and v^T p are formed from per-warp partial sums written in the
-// preceding phase.  On return dd, ee hold the tridiagonal, tau the reflector
-// scalars and column k of W below the diagonal the reflector v_k, which is
-// also written to hv[k n + i] (i < n - k - 1) when hv is given.  v, p: n df of
-// scratch each; red_sig, red_vp: 32 per-warp partial sums each.
-__device__ void syev_tridiagonalise(int n, df* W, long long LD, df* v, df* p, df* dd, df* ee, df* tau,
-                                    df_acc* red_sig, df_acc* red_vp, df* hv) {
-  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
-  // sigma partials of column 0 (rows 2..n-1)
-  {
-    df_acc a = acc_zero();
-    for (int i = 2 + warp; i < n; i += nw)
-      if (lane == 0) a.fma(W[i * LD], W[i * LD]);
-    if (lane == 0) red_sig[warp] = a;
-  }
-  __syncthreads();
-  for (int k = 0; k + 2 < n; ++k) {
-    const int m = n - k - 1;
-    df_acc sa = lane < nw ? red_sig[lane] : acc_zero();
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) sa.merge(shfl_xor_acc(sa, o));
-    const df sigma = sa.value();
-    const df x0 = W[(k + 1) * LD + k];
-    if (sigma.hi == 0.f) {
-      if (tid == 0) {
-        tau[k] = df{0.f, 0.f};
-        dd[k] = W[k * LD + k];
-        ee[k] = x0;
-      }
-      // partials of the next column, unchanged by this step
-      __syncthreads();
-      df_acc a = acc_zero();
-      for (int i = k + 3 + warp; i < n; i += nw)
-        if (lane == 0) a.fma(W[i * LD + k + 1], W[i * LD + k + 1]);
-      if (lane == 0) red_sig[warp] = a;
-      __syncthreads();
-      continue;
-    }
-    const df nrm = df_sqrt(df_add(df_mul(x0, x0), sigma));
-    const df alpha = df_lt0(x0) ? nrm : df_neg(nrm);
-    const df v0 = df_sub(x0, alpha);
-    const df vtv = df_add(sigma, df_mul(v0, v0));
-    const df t = df_div(df{2.f, 0.f}, vtv);
-    for (int i = tid; i < m; i += nt) v[i] = (i == 0) ? v0 : W[(k + 1 + i) * LD + k];
-    if (tid == 0) {
-      tau[k] = t;
-      dd[k] = W[k * LD + k];
-      ee[k] = alpha;
-    }
-    __syncthreads();  // (1) v complete
-    // p = t * W22 v, and per-warp partials of v^T p; column k keeps v for the back-transformation
-    {
-      df_acc pv = acc_zero();
-      for (int i = warp; i < m; i += nw) {
-        df_acc b0 = acc_zero(), b1 = acc_zero();
-        const df* row = W + (k + 1 + i) * LD + (k + 1);
-        int j = lane;
-        for (; j + 32 < m; j += 64) {
-          const df r0 = row[j], r1 = row[j + 32];
-          const df v0j = v[j], v1j = v[j + 32];
-          b0.fma(r0, v0j);
-          b1.fma(r1, v1j);
-        }
-        if (j < m) b0.fma(row[j], v[j]);
-        b0.merge(b1);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) b0.merge(shfl_xor_acc(b0, o));
-        if (lane == 0) {
-          const df pi = df_mul(t, b0.value());
-          p[i] = pi;
-          pv.fma(v[i], pi);
-        }
-      }
-      if (lane == 0) red_vp[warp] = pv;
-      for (int i = tid; i < m; i += nt) W[(k + 1 + i) * LD + k] = v[i];
-      if (hv != nullptr)
-        for (int i = tid; i < m; i += nt) hv[static_cast<long long>(k) * n + i] = v[i];
-    }
-    __syncthreads();  // (2) p and v^T p partials complete
-    {
-      df_acc c = lane < nw ? red_vp[lane] : acc_zero();
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) c.merge(shfl_xor_acc(c, o));
-      const df kc = df_mul(df_mul_f(t, 0.5f), c.value());
-      for (int i = tid; i < m; i += nt) p[i] = df_sub(p[i], df_mul(kc, v[i]));  // w
-    }
-    __syncthreads();  // (3) w complete
-    // W22 -= v w^T + w v^T over whole rows (coalesced; no mirrored column writes):
-    // entry (r, c) takes its two products in the order of (max, min), so both
-    // triangles stay bitwise equal.  Lane 0 of each row also accumulates the next
-    // column's norm (rows 2.. of the trailing block)
-    {
-      df_acc sg = acc_zero();
-      for (int i = warp; i < m; i += nw) {
-        const df vi = v[i], wi = p[i];
-        df* rowi = W + (k + 1 + i) * LD + (k + 1);
+// 1 / b with a relative error of about 2^-48 in a chain of ~70 cycles (df_recip: 220, df_div: 650):
+// the remainder 1 - b.hi r of the float32 reciprocal is exact to its last bit as one fused multiply-add, so
+// r (1 + e + e^2) needs no float-float operation before the final sum.
+__device__ __forceinline__ df df_recip_short(df b) {
+  const float r = __frcp_rn(b.hi);
+  const float e = __fmaf_rn(-b.lo, r, __fmaf_rn(-b.hi, r, 1.f));
+  return fast_two_sum(r, __fmul_rn(r, __fmaf_rn(e, e, e)));
+}
+
+// Inverse iteration in float-float for the shift sg of index j where it is in no
+// cluster of nearly equal shifts, by one warp: T - sg I = L D L^T (pivots kept at least pv in
+// magnitude) and the solves from a fixed start vector, the recurrences by lane 0 and
+// everything that is element by element by the lanes.  `solves` is 2 where the
+// neighbouring shifts are more than 1e-3 ||T|| away, else 3: each solve multiplies the other
+// directions by (shift error, below 1e-14 ||T||) / gap, so two leave less than 1e-20 of them.
+// Element i of the arrays at [i ld].
+__device__ void syev_inverse_iteration_warp(int j, int solves, df sg, const df* dd, const df* ee, int n, float pv,
+                                            df* dinv, df* lm, df* Z, long long ld) {
+  const int lane = threadIdx.x & 31;
+  if (lane == 0) {
+    df d = df_sub(dd[0], sg);
+    if (fabsf(d.hi) < pv) d = df{df_lt0(d) ? -pv : pv, 0.f};
+    df di = df_recip_short(d);
+    dinv[0] = di;
 #pragma unroll 2
-        for (int j = lane; j < m; j += 32) {
-          df_acc u0 = acc_zero();
-          if (j <= i) {
-            u0.fma(vi, p[j]);
-            u0.fma(wi, v[j]);
-          } else {
-            u0.fma(v[j], wi);
-            u0.fma(p[j], vi);
-          }
-          const df n0 = df_sub(rowi[j], u0.value());
-          rowi[j] = n0;
-          if (j == 0 && i >= 2) sg.fma(n0, n0);
-        }
-      }
-      if (lane == 0) red_sig[warp] = sg;
-    }
-    __syncthreads();  // (4) trailing block and next-column partials complete
-  }
-  if (tid == 0) {
-    if (n >= 2) {
-      dd[n - 2] = W[(n - 2) * LD + (n - 2)];
-      dd[n - 1] = W[(n - 1) * LD + (n - 1)];
-      ee[n - 2] = W[(n - 1) * LD + (n - 2)];
-      tau[n - 2] = df{0.f, 0.f};
-    } else {
-      dd[0] = W[0];
-    }
-    if (n >= 1) tau[n - 1] = df{0.f, 0.f};
-  }
-  __syncthreads();
-}
-
-// Gershgorin interval of the tridiagonal (float32 diagonal sd, squared
-// off-diagonal se2), padded, by one thread: sf = {lower, upper, ||T|| bound,
-// pivot floor of the Sturm recurrences}.
-__device__ void syev_bounds(const float* sd, const float* se2, int n, float* sf) {
-  float gl = 3.0e38f, gu = -3.0e38f, emax2 = 0.f;
-  for (int i = 0; i < n; ++i) {
-    const float r = (i > 0 ? sqrtf(se2[i - 1]) : 0.f) + (i + 1 < n ? sqrtf(se2[i]) : 0.f);
-    gl = fminf(gl, sd[i] - r);
-    gu = fmaxf(gu, sd[i] + r);
-    if (i + 1 < n) emax2 = fmaxf(emax2, se2[i]);
-  }
-  const float tn = fmaxf(fabsf(gl), fabsf(gu));
-  const float pad = 2.0e-6f * tn + 1.0e-30f;
-  sf[0] = gl - pad;
-  sf[1] = gu + pad;
-  sf[2] = tn;
-  sf[3] = fmaxf(1.0e-30f, 1.0e-35f * fmaxf(emax2, 1.f));
-}
-
-// float32 bracket of the (j+1)-th smallest eigenvalue by one warp: 32-point multisection, 33x narrower per round
-// (Golub & Van Loan 8.4.1), until the float32 points stop separating.
-__device__ float syev_multisect(int j, const float* sd, const float* se2, int n, float gl, float gu, float pivmin) {
-  const int lane = threadIdx.x & 31;
-  float lo = gl, hi = gu;
-  for (int round = 0; round < 40; ++round) {
-    const float mid = 0.5f * (lo + hi);
-    if (mid <= lo || mid >= hi) break;
-    const float x = lo + (hi - lo) * (static_cast<float>(lane + 1) * (1.f / 33.f));
-    const unsigned above = __ballot_sync(0xffffffffu, sturm_count(sd, se2, n, x, pivmin) > j);
-    const int l1 = above ? __ffs(above) - 1 : 32;  // first point with more than j eigenvalues below
-    const float xlo = __shfl_sync(0xffffffffu, x, l1 > 0 ? l1 - 1 : 0);
-    const float xhi = __shfl_sync(0xffffffffu, x, l1 < 32 ? l1 : 31);
-    if (l1 > 0) lo = fmaxf(lo, xlo);
-    if (l1 < 32) hi = fminf(hi, xhi);
-  }
-  return 0.5f * (lo + hi);
-}
-
-// Refine the float32 shift s0 of index j with float-float Sturm counts (one
-// warp; ee2 holds e_i^2).  The float32 counts can be off by ~n 2^-24 ||T||,
-// far more than the gaps inside a graded spectrum; with float-float shifts the
-// inverse iteration separates eigenvalues down to ~1e-9 ||T|| apart on its
-// own.  The bracket is first widened until its float-float counts enclose
-// index j, then 32-point multisection shrinks it 33x per round.  Returns the
-// midpoint of the final bracket (the same on every lane).
-__device__ df syev_refine_shift(int j, float s0, const df* dd, const df* ee2, int n, float gl, float gu,
-                                float tnorm, float pivmin) {
-  const int lane = threadIdx.x & 31;
-  float w = 1.0e-4f * tnorm + 1.0e-6f * fabsf(s0) + pivmin;
-  df lo = df{s0 - w, 0.f}, hi = df{s0 + w, 0.f};
-  for (int attempt = 0; attempt < 12; ++attempt) {
-    int c = 0;
-    if (lane < 2) c = sturm_count_df(dd, ee2, n, lane == 0 ? lo : hi, pivmin);
-    const int clo = __shfl_sync(0xffffffffu, c, 0), chi = __shfl_sync(0xffffffffu, c, 1);
-    if (clo <= j && chi > j) break;
-    w *= 4.f;
-    if (attempt == 11) {
-      lo = df{gl, 0.f};
-      hi = df{gu, 0.f};
-    } else {
-      if (clo > j) lo = df{s0 - w, 0.f};
-      if (chi <= j) hi = df{s0 + w, 0.f};
-    }
-  }
-  const float tol = 1.0e-14f * tnorm + pivmin;
-  for (int round = 0; round < 12; ++round) {
-    const df width = df_sub(hi, lo);
-    if (!(width.hi > tol)) break;
-    const df x = df_add(lo, df_mul_f(width, static_cast<float>(lane + 1) * (1.f / 33.f)));
-    const unsigned above = __ballot_sync(0xffffffffu, sturm_count_df(dd, ee2, n, x, pivmin) > j);
-    const int l1 = above ? __ffs(above) - 1 : 32;  // first point with more than j eigenvalues below
-    const float lhi = __shfl_sync(0xffffffffu, x.hi, l1 > 0 ? l1 - 1 : 0);
-    const float llo = __shfl_sync(0xffffffffu, x.lo, l1 > 0 ? l1 - 1 : 0);
-    const float hhi = __shfl_sync(0xffffffffu, x.hi, l1 < 32 ? l1 : 31);
-    const float hlo = __shfl_sync(0xffffffffu, x.lo, l1 < 32 ? l1 : 31);
-    if (l1 > 0) lo = df{lhi, llo};
-    if (l1 < 32) hi = df{hhi, hlo};
-  }
-  return df_mul_f(df_add(lo, hi), 0.5f);
-}
-
-// Gap between consecutive refined shifts, compared in float32 against the
-// cluster and group thresholds below.
-__device__ __forceinline__ float shift_gap(const df* shd, int j) {
-  return j > 0 ? df_float(df_sub(shd[j], shd[j - 1])) : 3.0e38f;
-}
-
-// Inverse iteration in float-float for the shift sg of index j, one thread:
-// T - sg I = L D L^T (pivots kept at least pv in magnitude), three solves from
-// a fixed start vector, each followed by Gram-Schmidt against the finished
-// members c0 .. jj-1 of its cluster and a normalisation.  Element i of the
-// vector, of 1/d and of l is at [i ld + jj] of Z, dinv and lm.
-__device__ void syev_inverse_iteration(int j, int jj, int c0, df sg, const df* dd, const df* ee, int n, df pv,
-                                       df* dinv, df* lm, df* Z, long long ld) {
-  df d = df_sub(dd[0], sg);
-  if (fabsf(d.hi) < pv.hi) d = df_lt0(d) ? df_neg(pv) : pv;
-  df di = df_div(df{1.f, 0.f}, d);
-  dinv[jj] = di;
-  for (int i = 1; i < n; ++i) {
-    const df e = ee[i - 1];
-    const df l = df_mul(e, di);
-    lm[(i - 1) * ld + jj] = l;
-    d = df_sub(df_sub(dd[i], sg), df_mul(l, e));
-    if (fabsf(d.hi) < pv.hi) d = df_lt0(d) ? df_neg(pv) : pv;
-    di = df_div(df{1.f, 0.f}, d);
-    dinv[i * ld + jj] = di;
-  }
-  // start vector
-  for (int i = 0; i < n; ++i) Z[i * ld + jj] = df{1.f + 0.37f * (float)((i * 7 + j * 13) % 11) / 11.f, 0.f};
-  for (int it = 0; it < 3; ++it) {
-    // L w = x ; z = D^-1 w ; L^T y = z
-    df prev = Z[jj];
     for (int i = 1; i < n; ++i) {
-      prev = df_sub(Z[i * ld + jj], df_mul(lm[(i - 1) * ld + jj], prev));
-      Z[i * ld + jj] = prev;
+      const df e = ee[i - 1];
+      const df l = df_mul(e, di);
+      lm[(i - 1) * ld] = l;
+      d = df_sub(df_sub(dd[i], sg), df_mul(l, e));
+      if (fabsf(d.hi) < pv) d = df{df_lt0(d) ? -pv : pv, 0.f};
+      di = df_recip_short(d);
+      dinv[i * ld] = di;
     }
-    df nxt = df_mul(Z[(n - 1) * ld + jj], dinv[(n - 1) * ld + jj]);
-    Z[(n - 1) * ld + jj] = nxt;
-    for (int i = n - 2; i >= 0; --i) {
-      nxt = df_sub(df_mul(Z[i * ld + jj], dinv[i * ld + jj]), df_mul(lm[i * ld + jj], nxt));
-      Z[i * ld + jj] = nxt;
+  }
+  __syncwarp();
+  for (int i = lane; i < n; i += 32) Z[i * ld] = df{1.f + 0.37f * (float)((i * 7 + j * 13) % 11) / 11.f, 0.f};
+  __syncwarp();
+  for (int it = 0; it < solves; ++it) {
+    if (lane == 0) {
+      df prev = Z[0];
+#pragma unroll 4
+      for (int i = 1; i < n; ++i) {
+        prev = df_sub(Z[i * ld], df_mul(lm[(i - 1) * ld], prev));
+        Z[i * ld] = prev;
+      }
     }
-    // Gram-Schmidt against finished members of the cluster
-    for (int jp = c0; jp < jj; ++jp) {
-      df_acc dt = acc_zero();
-      for (int i = 0; i < n; ++i) dt.fma(Z[i * ld + jp], Z[i * ld + jj]);
-      const df dv = dt.value();
-      for (int i = 0; i < n; ++i) Z[i * ld + jj] = df_sub(Z[i * ld + jj], df_mul(dv, Z[i * ld + jp]));
+    __syncwarp();
+    for (int i = lane; i < n; i += 32) Z[i * ld] = df_mul(Z[i * ld], dinv[i * ld]);
+    __syncwarp();
+    if (lane == 0) {
+      df nxt = Z[(n - 1) * ld];
+#pragma unroll 4
+      for (int i = n - 2; i >= 0; --i) {
+        nxt = df_sub(Z[i * ld], df_mul(lm[i * ld], nxt));
+        Z[i * ld] = nxt;
+      }
     }
-    // normalise (scale first by the largest entry to stay in range)
+    __syncwarp();
     float amax = 0.f;
-    for (int i = 0; i < n; ++i) amax = fmaxf(amax, fabsf(Z[i * ld + jj].hi));
-    const float sc1 = amax > 0.f ? 1.f / amax : 1.f;
+    for (int i = lane; i < n; i += 32) amax = fmaxf(amax, fabsf(Z[i * ld].hi));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+    const float r = amax > 0.f ? exp2f(-floorf(log2f(amax))) : 1.f;  // exact scaling
     df_acc dn = acc_zero();
-    for (int i = 0; i < n; ++i) {
-      const df z = df_mul_f(Z[i * ld + jj], sc1);
-      Z[i * ld + jj] = z;
+    for (int i = lane; i < n; i += 32) {
+      const df z = df{Z[i * ld].hi * r, Z[i * ld].lo * r};
+      Z[i * ld] = z;
       dn.fma(z, z);
     }
-    const df inv = df_div(df{1.f, 0.f}, df_sqrt(dn.value()));
-    for (int i = 0; i < n; ++i) Z[i * ld + jj] = df_mul(Z[i * ld + jj], inv);
+    if (it + 1 == solves) {
+      const df inv = shfl_df(df_div(df{1.f, 0.f}, df_sqrt(warp_acc_sum(dn).value())), 0);
+      for (int i = lane; i < n; i += 32) Z[i * ld] = df_mul(Z[i * ld], inv);
+    }
+    __syncwarp();
   }
 }
 
-// A vector alone in its group, one thread: its Rayleigh quotient with T goes
+// A vector alone in its group, one warp: its Rayleigh quotient with T goes
 // to *eval and the vector, normalised, to Zn (element i at [i ldn]).  Z holds
 // element i at [i ldz].
 __device__ void syev_single(const df* Z, long long ldz, const df* dd, const df* ee, int n, df* Zn, long long ldn,
                             double* eval) {
+  const int lane = threadIdx.x & 31;
   df_acc sq = acc_zero(), hq = acc_zero();
-  for (int i = 0; i < n; ++i) {
+  for (int i = lane; i < n; i += 32) {
     const df z = Z[i * ldz];
     df_acc tz = acc_zero();
     tz.fma(dd[i], z);
@@ -450,308 +213,11 @@ __device__ void syev_single(const df* Z, long long ldz, const df* dd, const df* 
     sq.fma(z, z);
     hq.fma(z, tz.value());
   }
-  const df sv = sq.value();
+  const df sv = shfl_df(warp_acc_sum(sq).value(), 0);
+  const df hv = shfl_df(warp_acc_sum(hq).value(), 0);
   const df inv = df_div(df{1.f, 0.f}, df_sqrt(sv));
-  for (int i = 0; i < n; ++i) Zn[i * ldn] = df_mul(Z[i * ldz], inv);
-  *eval = df_to_double(df_div(hq.value(), sv));
-}
-
-// Rayleigh-Ritz clean-up of one group of G >= 2 vectors by the whole block.
-// The group's shifts are more than 1e-4 ||T|| from every other group's, so each
-// vector's error outside its own group's span is below ~4e-11, and a
-// Rayleigh-Ritz step on the span (S = Z_g^T Z_g, Hq = Z_g^T T Z_g) restores
-// working accuracy: S = L L^T, C = L^-1 Hq L^-T by parallel cyclic Jacobi,
-// vectors Z_g L^-T Q in ascending order.  Column c of the group is at
-// Z[i ldz + c] and goes to Zn[i ldn + c], its eigenvalue to evals[c].  rrw:
-// 4 G^2 df, perm: G ints, red, sf: block reduction scratch (shared).  TZ: n x G
-// df scratch with Z's row stride (T Z, formed once).  TA x TB: the register
-// tile of S and Hq per thread.
-template <int TA, int TB>
-__device__ void syev_group_rr(int G, const df* Z, long long ldz, const df* dd, const df* ee, int n, df* TZ,
-                              df* rrw, int* perm, df_acc* red, float* sf, df* Zn, long long ldn, double* evals) {
-  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
-  const long long N = n;
-  df* S = rrw;
-  df* Hq = rrw + G * G;
-  df* Qm = rrw + 2 * G * G;
-  df* Xm = rrw + 3 * G * G;
-  for (int i = warp; i < n; i += nw)
-    for (int c = lane; c < G; c += 32) {
-      df_acc tz = acc_zero();
-      tz.fma(dd[i], Z[i * ldz + c]);
-      if (i > 0) tz.fma(ee[i - 1], Z[(i - 1) * ldz + c]);
-      if (i + 1 < n) tz.fma(ee[i], Z[(i + 1) * ldz + c]);
-      TZ[i * ldz + c] = tz.value();
-    }
-  __syncthreads();
-  // S = Z^T Z and Hq = Z^T (T Z): the upper triangle by TA x TB tiles, one
-  // compensated sum per entry over the rows in order; the lower triangle mirrors it
-  {
-    // tile row ta starts at tile column (ta TA) / TB, the first that reaches the diagonal
-    const int na = (G + TA - 1) / TA, nbt = (G + TB - 1) / TB;
-    int ntile = 0;
-    for (int ta = 0; ta < na; ++ta) ntile += nbt - (ta * TA) / TB;
-    for (int tix = tid; tix < ntile; tix += nt) {
-      int ta = 0, rem = tix;
-      while (rem >= nbt - (ta * TA) / TB) {
-        rem -= nbt - (ta * TA) / TB;
-        ++ta;
-      }
-      const int a0 = ta * TA, b0 = ((ta * TA) / TB + rem) * TB;
-      df_acc sa[TA][TB], ha[TA][TB];
-#pragma unroll
-      for (int u = 0; u < TA; ++u)
-#pragma unroll
-        for (int v = 0; v < TB; ++v) sa[u][v] = ha[u][v] = acc_zero();
-      for (int i = 0; i < n; ++i) {
-        df za[TA], zb[TB], tb[TB];
-#pragma unroll
-        for (int u = 0; u < TA; ++u) za[u] = a0 + u < G ? Z[i * ldz + a0 + u] : df{0.f, 0.f};
-#pragma unroll
-        for (int v = 0; v < TB; ++v) {
-          const bool ib = b0 + v < G;
-          zb[v] = ib ? Z[i * ldz + b0 + v] : df{0.f, 0.f};
-          tb[v] = ib ? TZ[i * ldz + b0 + v] : df{0.f, 0.f};
-        }
-#pragma unroll
-        for (int u = 0; u < TA; ++u)
-#pragma unroll
-          for (int v = 0; v < TB; ++v) {
-            sa[u][v].fma(za[u], zb[v]);
-            ha[u][v].fma(za[u], tb[v]);
-          }
-      }
-#pragma unroll
-      for (int u = 0; u < TA; ++u)
-#pragma unroll
-        for (int v = 0; v < TB; ++v) {
-          const int a = a0 + u, b = b0 + v;
-          if (a <= b && b < G) {
-            S[a * G + b] = S[b * G + a] = sa[u][v].value();
-            Hq[a * G + b] = Hq[b * G + a] = ha[u][v].value();
-          }
-        }
-    }
-  }
-  __syncthreads();
-  // Cholesky S = L L^T in place (lower), right-looking
-  for (int kk = 0; kk < G; ++kk) {
-    if (tid == 0) S[kk * G + kk] = df_sqrt(S[kk * G + kk]);
-    __syncthreads();
-    const df piv = S[kk * G + kk];
-    for (int i = kk + 1 + tid; i < G; i += nt) S[i * G + kk] = df_div(S[i * G + kk], piv);
-    __syncthreads();
-    for (int idx = tid; idx < (G - kk - 1) * (G - kk - 1); idx += nt) {
-      const int i = kk + 1 + idx / (G - kk - 1), jj = kk + 1 + idx % (G - kk - 1);
-      if (jj <= i) S[i * G + jj] = df_sub(S[i * G + jj], df_mul(S[i * G + kk], S[jj * G + kk]));
-    }
-    __syncthreads();
-  }
-  // C = L^-1 Hq L^-T  (two column-parallel forward substitutions; each row's
-  // sum over the solved rows in four compensated chains)
-  for (int pass = 0; pass < 2; ++pass) {
-    df* out = pass == 0 ? Xm : Qm;
-    for (int col = tid; col < G; col += nt) {
-      for (int i = 0; i < G; ++i) {
-        const df rhs = (pass == 0) ? Hq[i * G + col] : Xm[col * G + i];
-        const df s = df_sub(rhs, dot4(S + i * G, 1, out + col, G, i).value());
-        out[i * G + col] = df_div(s, S[i * G + i]);
-      }
-    }
-    __syncthreads();
-  }
-  // Qm now holds C (symmetric); move it to Hq and set Qm = I
-  for (int idx = tid; idx < G * G; idx += nt) {
-    const int a0 = idx / G, b0 = idx % G;
-    const df cab = Qm[a0 * G + b0], cba = Qm[b0 * G + a0];
-    Hq[idx] = df_mul_f(df_add(cab, cba), 0.5f);
-  }
-  __syncthreads();
-  for (int idx = tid; idx < G * G; idx += nt) Qm[idx] = df{(idx / G == idx % G) ? 1.f : 0.f, 0.f};
-  __syncthreads();
-  // parallel cyclic Jacobi (round-robin pairing) on C, accumulating Q
-  {
-    const int np = (G + 1) & ~1;  // even player count; index G is a dummy
-    for (int sweep = 0; sweep < 12; ++sweep) {
-      // convergence test: largest off-diagonal entry against the largest diagonal one
-      float off = 0.f, dia = 0.f;
-      for (int idx = tid; idx < G * G; idx += nt) {
-        const int a0 = idx / G, b0 = idx % G;
-        const float x = fabsf(Hq[idx].hi);
-        if (a0 == b0) dia = fmaxf(dia, x); else off = fmaxf(off, x);
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        off = fmaxf(off, __shfl_xor_sync(0xffffffffu, off, o));
-        dia = fmaxf(dia, __shfl_xor_sync(0xffffffffu, dia, o));
-      }
-      if (lane == 0) {
-        red[warp].s = off;
-        red[warp].c = dia;
-      }
-      __syncthreads();
-      if (tid == 0) {
-        float o2 = 0.f, d2 = 0.f;
-        for (int w2 = 0; w2 < nw; ++w2) {
-          o2 = fmaxf(o2, red[w2].s);
-          d2 = fmaxf(d2, red[w2].c);
-        }
-        sf[0] = o2;
-        sf[1] = d2;
-      }
-      __syncthreads();
-      const float offmax = sf[0], diamax = sf[1];
-      __syncthreads();
-      if (!(offmax > 1.0e-15f * fmaxf(diamax, 1.0e-30f))) break;
-      for (int r = 0; r < np - 1; ++r) {
-        // pair t: players (a, b) of the round-robin schedule
-        for (int t = tid; t < np / 2; t += nt) {
-          int a0 = (t == 0) ? 0 : 1 + (t - 1 + r) % (np - 1);
-          int b0 = 1 + (np - 2 - t + r) % (np - 1);
-          if (a0 > b0) {
-            const int tmpi = a0;
-            a0 = b0;
-            b0 = tmpi;
-          }
-          df cs = df{1.f, 0.f}, sn = df{0.f, 0.f};
-          if (b0 < G) {
-            const df apq = Hq[a0 * G + b0];
-            const df app = Hq[a0 * G + a0], aqq = Hq[b0 * G + b0];
-            // skip entries already below the float-float resolution of the diagonal
-            const float thr = 1.0e-17f * (sqrtf(fabsf(app.hi)) * sqrtf(fabsf(aqq.hi))) + 1.0e-37f;
-            if (fabsf(apq.hi) > thr) {
-              // theta = (aqq - app) / (2 apq); t = sign(theta) / (|theta| + sqrt(theta^2 + 1)),
-              // and t = 1 / (2 theta) once theta^2 would leave the float range
-              const df th = df_div(df_sub(aqq, app), df_mul_f(apq, 2.f));
-              df tt;
-              if (fabsf(th.hi) > 1.0e12f) {
-                tt = df_div(df{0.5f, 0.f}, th);
-              } else {
-                const df rt = df_sqrt(df_add(df_mul(th, th), df{1.f, 0.f}));
-                tt = df_div(df{1.f, 0.f}, df_add(df_abs(th), rt));
-                if (df_lt0(th)) tt = df_neg(tt);
-              }
-              cs = df_div(df{1.f, 0.f}, df_sqrt(df_add(df_mul(tt, tt), df{1.f, 0.f})));
-              sn = df_mul(tt, cs);
-            }
-          }
-          // stash rotation in Xm row 0..np/2 (cols 0..3)
-          Xm[t * 4 + 0] = cs;
-          Xm[t * 4 + 1] = sn;
-          reinterpret_cast<int*>(&Xm[t * 4 + 2])[0] = a0;
-          reinterpret_cast<int*>(&Xm[t * 4 + 3])[0] = b0;
-        }
-        __syncthreads();
-        // C <- J^T C J by 2 x 2 blocks (pair s, pair t), s <= t, the lower
-        // triangle mirrored; the rows of each block turn first, then its columns.
-        // The triangle of pair blocks is folded (row s with row P - 1 - s) so
-        // that every thread gets the same share.  Q <- Q J alongside.
-        {
-          const int P = np / 2, half = (P + 1) / 2;
-          for (int idx = tid; idx < half * (P + 1); idx += nt) {
-            const int fr = idx / (P + 1), cc = idx - fr * (P + 1);
-            int ps, pt;
-            if (cc < P - fr) {
-              ps = fr;
-              pt = fr + cc;
-            } else {
-              ps = P - 1 - fr;
-              if (ps == fr) continue;
-              pt = ps + (cc - (P - fr));
-            }
-            const int as = reinterpret_cast<const int*>(&Xm[ps * 4 + 2])[0];
-            const int bs = reinterpret_cast<const int*>(&Xm[ps * 4 + 3])[0];
-            const int at = reinterpret_cast<const int*>(&Xm[pt * 4 + 2])[0];
-            const int bt = reinterpret_cast<const int*>(&Xm[pt * 4 + 3])[0];
-            const df css = Xm[ps * 4 + 0], sns = Xm[ps * 4 + 1];
-            const df cst = Xm[pt * 4 + 0], snt = Xm[pt * 4 + 1];
-            const bool rs = bs < G, rt = bt < G;
-            const df zero = df{0.f, 0.f};
-            df x00 = Hq[as * G + at], x01 = rt ? Hq[as * G + bt] : zero;
-            df x10 = rs ? Hq[bs * G + at] : zero, x11 = (rs && rt) ? Hq[bs * G + bt] : zero;
-            if (rs) {
-              const df y00 = df_sub(df_mul(css, x00), df_mul(sns, x10));
-              const df y10 = df_add(df_mul(sns, x00), df_mul(css, x10));
-              const df y01 = df_sub(df_mul(css, x01), df_mul(sns, x11));
-              const df y11 = df_add(df_mul(sns, x01), df_mul(css, x11));
-              x00 = y00;
-              x10 = y10;
-              x01 = y01;
-              x11 = y11;
-            }
-            if (rt) {
-              const df y00 = df_sub(df_mul(cst, x00), df_mul(snt, x01));
-              const df y01 = df_add(df_mul(snt, x00), df_mul(cst, x01));
-              const df y10 = df_sub(df_mul(cst, x10), df_mul(snt, x11));
-              const df y11 = df_add(df_mul(snt, x10), df_mul(cst, x11));
-              x00 = y00;
-              x01 = y01;
-              x10 = y10;
-              x11 = y11;
-            }
-            if (ps == pt) {
-              // diagonal block: (as, bs) and (bs, as) take the same value
-              Hq[as * G + as] = x00;
-              if (rs) {
-                Hq[as * G + bs] = Hq[bs * G + as] = x01;
-                Hq[bs * G + bs] = x11;
-              }
-            } else {
-              Hq[as * G + at] = Hq[at * G + as] = x00;
-              if (rt) Hq[as * G + bt] = Hq[bt * G + as] = x01;
-              if (rs) Hq[bs * G + at] = Hq[at * G + bs] = x10;
-              if (rs && rt) Hq[bs * G + bt] = Hq[bt * G + bs] = x11;
-            }
-          }
-          for (int t = warp; t < P; t += nw) {
-            const int a0 = reinterpret_cast<const int*>(&Xm[t * 4 + 2])[0];
-            const int b0 = reinterpret_cast<const int*>(&Xm[t * 4 + 3])[0];
-            if (b0 >= G) continue;
-            const df cs = Xm[t * 4 + 0], sn = Xm[t * 4 + 1];
-            for (int row = lane; row < G; row += 32) {
-              const df x = Qm[row * G + a0], y = Qm[row * G + b0];
-              Qm[row * G + a0] = df_sub(df_mul(cs, x), df_mul(sn, y));
-              Qm[row * G + b0] = df_add(df_mul(sn, x), df_mul(cs, y));
-            }
-          }
-        }
-        __syncthreads();
-      }
-    }
-  }
-  // order eigenvalues ascending (selection by rank; ties broken by index); the identity first, so that
-  // perm holds valid columns even when a NaN leaves ranks unassigned
-  for (int j = tid; j < G; j += nt) perm[j] = j;
-  __syncthreads();
-  for (int j = tid; j < G; j += nt) {
-    const df lj = Hq[j * G + j];
-    int rank = 0;
-    for (int i = 0; i < G; ++i) {
-      const df li = Hq[i * G + i];
-      const df dlt = df_sub(li, lj);
-      if (df_lt0(dlt) || ((dlt.hi == 0.f && dlt.lo == 0.f) && i < j)) ++rank;
-    }
-    perm[rank] = j;
-  }
-  __syncthreads();
-  // Xm = L^-T Q  (back substitution per column)
-  for (int col = tid; col < G; col += nt) {
-    for (int i = G - 1; i >= 0; --i) {
-      const df s = df_sub(Qm[i * G + col], dot4(S + (i + 1) * G + i, G, Xm + (i + 1) * G + col, G, G - 1 - i).value());
-      Xm[i * G + col] = df_div(s, S[i * G + i]);
-    }
-  }
-  __syncthreads();
-  // group eigenvectors Zn[:, c] = Z_g Xm[:, perm[c]] (ascending within the group)
-  for (long long idx = tid; idx < N * G; idx += nt) {
-    const int i = static_cast<int>(idx / G), c = static_cast<int>(idx % G);
-    const int src = perm[c];
-    df_acc sa = acc_zero();
-    for (int kk = 0; kk < G; ++kk) sa.fma(Z[i * ldz + kk], Xm[kk * G + src]);
-    Zn[i * ldn + c] = sa.value();
-  }
-  for (int c = tid; c < G; c += nt) evals[c] = df_to_double(Hq[perm[c] * G + perm[c]]);
-  __syncthreads();
+  for (int i = lane; i < n; i += 32) Zn[i * ldn] = df_mul(Z[i * ldz], inv);
+  if (lane == 0) *eval = df_to_double(df_div(hv, sv));
 }
 
 // Global workspace: W (n x ldw df) unless it fits in shared memory, the
@@ -759,40 +225,12 @@ __device__ void syev_group_rr(int G, const df* Z, long long ldz, const df* dd, c
 // (df, nwant) and their bounds (4 floats), the factors and working vectors of
 // groups too wide for shared memory (fac: 3 n nwant df) and the tridiagonal
 // eigenvectors Zg (n x nwant df).
-constexpr int kSvWarps = 4;  // shifts per block of k_syev_vals
+constexpr int kSvThreads = 128;  // points per round of k_syev_vals
 constexpr int kSvecThreads = 512;
-constexpr int kSbWarps = 8;  // eigenvectors per block of k_syev_back
-constexpr int kSbChunk = 8;  // reflectors staged per barrier in k_syev_back
+constexpr int kSbWarps = 4;  // eigenvectors per block of k_syev_back
+constexpr int kSbChunk = 8;  // reflectors applied together in k_syev_back
 
-// Tridiagonalisation, one block: W in shared memory when `inshared`, else the
-// global Wg.  Writes dd, ee, tau and the reflectors hv to global memory.
-__global__ void __launch_bounds__(kSyThreads) k_syev_tri(int n, int ldw, int inshared, const double* __restrict__ H,
-                                                         df* __restrict__ Wg, df* __restrict__ hv,
-                                                         df* __restrict__ dd_g, df* __restrict__ ee_g,
-                                                         df* __restrict__ tau_g, const int* __restrict__ skip) {
-  if (skip != nullptr && *skip != 0) return;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  df* v = reinterpret_cast<df*>(smem_raw);
-  df* p = v + n;
-  df* dd = p + n;
-  df* ee = dd + n;
-  df* tau = ee + n;
-  const size_t off = (5 * sizeof(df) * static_cast<size_t>(n) + 15) & ~static_cast<size_t>(15);
-  df* W = inshared ? reinterpret_cast<df*>(smem_raw + off) : Wg;
-  __shared__ df_acc red_sig[32], red_vp[32];
-  const int tid = threadIdx.x, nt = blockDim.x;
-  const long long N = n, LD = ldw;
-  for (long long i = tid; i < N * N; i += nt) W[(i / N) * LD + (i % N)] = df_from_double(H[i]);
-  __syncthreads();
-  syev_tridiagonalise(n, W, LD, v, p, dd, ee, tau, red_sig, red_vp, hv);
-  for (int i = tid; i < n; i += nt) {
-    dd_g[i] = dd[i];
-    tau_g[i] = tau[i];
-    if (i + 1 < n) ee_g[i] = ee[i];
-  }
-}
-
-// The same tridiagonalisation by a thread-block cluster of 16 CTAs, row i of W in CTA
+// Householder tridiagonalisation by a thread-block cluster of 16 CTAs, row i of W in CTA
 // i % 16's shared memory (dealt cyclically, so the shrinking trailing block stays
 // spread over all of them).  A step is bound by the latency of its chain more than by
 // its work, so it exchanges only what the next link needs:
@@ -821,12 +259,6 @@ constexpr int kTriMaxN = kTriCluster * kTriRowWarps * kTriRows;
 static_assert(kTriMaxN <= 32 * kTriRowWarps && kTriRowWarps == kTriCluster && kTriMaxN / kTriCluster <= 32,
               "one thread per element of p, one warp per destination, one lane per own row");
 constexpr int kTriOneBlock = 40;  // below this size one block's barriers are cheaper
-
-__device__ __forceinline__ df_acc warp_acc_sum(df_acc a) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) a.merge(shfl_xor_acc(a, o));
-  return a;
-}
 
 // w - (v_i w_j + v_j w_i): compensated products, symmetric in (i, j) bit for bit
 __device__ __forceinline__ df rank2_update(df w, df vi, df wi, df vj, df wj) {
@@ -997,53 +429,122 @@ __global__ void __launch_bounds__(kTriThreads) k_syev_tri_cl(int n, int ldw, con
   cl.sync();  // no CTA leaves while another may still write into its shared memory
 }
 
-// The refined shifts, one warp each (kSvWarps per block): float32 multisection
-// then float-float refinement.  Block 0 also writes the bounds.  Shared: dd,
-// ee2 (df, n each), sd, se2 (float, n each).
-__global__ void __launch_bounds__(32 * kSvWarps) k_syev_vals(int n, int nwant, const df* __restrict__ dd_g,
-                                                             const df* __restrict__ ee_g, df* __restrict__ shd,
-                                                             float* __restrict__ bounds,
-                                                             const int* __restrict__ skip) {
+// The shifts, one block each: a multisection by Sturm counts at kSvThreads points per
+// round, three rounds in float32, then in float-float from a bracket of 1e-4 ||T||
+// around the float32 value (float32 counts can be off by far more than the gaps of a
+// graded spectrum; with float-float shifts the inverse iteration separates
+// eigenvalues down to ~1e-9 ||T|| on its own) until it is 1e-14 ||T|| wide: every round
+// counts at both ends too and moves the bracket outward when they do not
+// enclose the index.  Bound by the latency of a count's n-step chain, so the
+// points per round are many (127x narrower per round, five rounds) and a block
+// has one warp per scheduler.  One warp per shift with 33x per round and the
+// quotient recurrence took 478 us for 128 of 256 (129 now).  The grid covers one shift more than wanted (the
+// vectors' gaps to it decide on their solves).  Block 0 also writes the bounds: Gershgorin interval,
+// ||T|| and the pivot floor.  Shared: d, e^2 scaled by a power of two to ||T|| <= 1
+// (df, n each).
+__global__ void __launch_bounds__(kSvThreads) k_syev_vals(int n, const df* __restrict__ dd_g,
+                                                          const df* __restrict__ ee_g, df* __restrict__ shd,
+                                                          float* __restrict__ bounds,
+                                                          const int* __restrict__ skip) {
   if (skip != nullptr && *skip != 0) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  df* dd = reinterpret_cast<df*>(smem_raw);
-  df* ee2 = dd + n;
-  float* sd = reinterpret_cast<float*>(ee2 + n);
-  float* se2 = sd + n;
-  __shared__ float sf[4];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  for (int i = tid; i < n; i += blockDim.x) {
-    const df d = dd_g[i];
-    dd[i] = d;
-    sd[i] = df_float(d);
-    if (i + 1 < n) {
-      const df e = ee_g[i];
-      const float ef = df_float(e);
-      se2[i] = ef * ef;
-      ee2[i] = df_mul(e, e);
-    }
+  df* d = reinterpret_cast<df*>(smem_raw);
+  df* e2 = d + n;
+  constexpr int NW = kSvThreads / 32;
+  __shared__ float red[3][NW];
+  __shared__ int fa[2][NW];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, j = blockIdx.x;
+  float gl = 3.0e38f, gu = -3.0e38f, emax2 = 0.f;
+  for (int i = tid; i < n; i += kSvThreads) {
+    const df di = dd_g[i];
+    d[i] = di;
+    const float x = df_float(di);
+    const float el = i > 0 ? fabsf(df_float(ee_g[i - 1])) : 0.f;
+    const df er = i + 1 < n ? ee_g[i] : df{0.f, 0.f};
+    const float ef = fabsf(df_float(er));
+    e2[i] = er;
+    gl = fminf(gl, x - (el + ef));
+    gu = fmaxf(gu, x + (el + ef));
+    emax2 = fmaxf(emax2, ef * ef);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    gl = fminf(gl, __shfl_xor_sync(0xffffffffu, gl, o));
+    gu = fmaxf(gu, __shfl_xor_sync(0xffffffffu, gu, o));
+    emax2 = fmaxf(emax2, __shfl_xor_sync(0xffffffffu, emax2, o));
+  }
+  if (lane == 0) {
+    red[0][warp] = gl;
+    red[1][warp] = gu;
+    red[2][warp] = emax2;
   }
   __syncthreads();
-  if (tid == 0) syev_bounds(sd, se2, n, sf);
+#pragma unroll
+  for (int w = 0; w < NW; ++w) {
+    gl = fminf(gl, red[0][w]);
+    gu = fmaxf(gu, red[1][w]);
+    emax2 = fmaxf(emax2, red[2][w]);
+  }
+  const float tnorm = fmaxf(fabsf(gl), fabsf(gu));
+  const float pad = 2.0e-6f * tnorm + 1.0e-30f;
+  gl -= pad;
+  gu += pad;
+  if (j == 0 && tid == 0) {
+    bounds[0] = gl;
+    bounds[1] = gu;
+    bounds[2] = tnorm;
+    bounds[3] = fmaxf(1.0e-30f, 1.0e-35f * fmaxf(emax2, 1.f));
+  }
+  const int ex = tnorm > 0.f ? min(126, max(-126, ilogbf(tnorm) + 1)) : 0;
+  const float sc = exp2f(static_cast<float>(-ex)), un = exp2f(static_cast<float>(ex));
+  for (int i = tid; i < n; i += kSvThreads) {
+    const df di = d[i], er = df{e2[i].hi * sc, e2[i].lo * sc};
+    d[i] = df{di.hi * sc, di.lo * sc};
+    e2[i] = df_mul(er, er);
+  }
   __syncthreads();
-  if (blockIdx.x == 0 && tid < 4) bounds[tid] = sf[tid];
-  const int j = blockIdx.x * kSvWarps + warp;
-  if (j >= nwant) return;  // whole warps: no block barrier below
-  const float gl = sf[0], gu = sf[1], tnorm = sf[2], pivmin = sf[3];
-  const float s0 = syev_multisect(j, sd, se2, n, gl, gu, pivmin);
-  const df s = syev_refine_shift(j, s0, dd, ee2, n, gl, gu, tnorm, pivmin);
-  if (lane == 0) shd[j] = s;
-}
-
-// Bytes of shared memory k_syev_vecs keeps for a group of G vectors: d, e
-// (2n df), cluster data (2G ints), perm (G ints), and -- in shared memory when
-// they fit -- the factors and vectors (3 n G df) and the clean-up matrices (4 G^2 df).
-__host__ __device__ inline size_t syev_vecs_base(int n, int G) {
-  return (2 * sizeof(df) * static_cast<size_t>(n) + 3 * sizeof(int) * static_cast<size_t>(G) + 15) &
-         ~static_cast<size_t>(15);
-}
-__host__ __device__ inline size_t syev_vecs_work(int n, int G) {
-  return sizeof(df) * (3 * static_cast<size_t>(n) * G + 4 * static_cast<size_t>(G) * G);
+  int round = 0;
+  // the first of the block's points with more than j eigenvalues below (kSvThreads if none)
+  auto first_above = [&](bool above) {
+    const unsigned m = __ballot_sync(0xffffffffu, above);
+    const int buf = round++ & 1;
+    if (lane == 0) fa[buf][warp] = m ? 32 * warp + __ffs(m) - 1 : kSvThreads;
+    __syncthreads();
+    int f = fa[buf][0];
+#pragma unroll
+    for (int w = 1; w < NW; ++w) f = min(f, fa[buf][w]);
+    return f;
+  };
+  float flo = gl * sc, fhi = gu * sc;
+  for (int r = 0; r < 3; ++r) {
+    const float h = (fhi - flo) * (1.f / (kSvThreads + 1));
+    const int f = first_above(sturm_count(d, e2, n, flo + h * static_cast<float>(tid + 1)) > j);
+    const float a = flo;
+    if (f > 0) flo = a + h * static_cast<float>(f);
+    if (f < kSvThreads) fhi = a + h * static_cast<float>(f + 1);
+  }
+  const float s0 = 0.5f * (flo + fhi);
+  df lo = df{s0 - 1.0e-4f, 0.f}, hi = df{s0 + 1.0e-4f, 0.f};
+  for (int r = 0; r < 16; ++r) {
+    const df width = df_sub(hi, lo);
+    if (!(width.hi > 7.0e-15f)) break;
+    auto point = [&](int t) { return df_add(lo, df_mul_f(width, static_cast<float>(t) * (1.f / (kSvThreads - 1)))); };
+    const int f = first_above(sturm_count_df(d, e2, n, point(tid)) > j);
+    if (f == 0) {
+      hi = lo;
+      lo = df_sub(lo, df_mul_f(width, 8.f));
+    } else if (f == kSvThreads) {
+      lo = point(kSvThreads - 1);
+      hi = df_add(lo, df_mul_f(width, 8.f));
+    } else {
+      hi = point(f);
+      lo = point(f - 1);
+    }
+  }
+  if (tid == 0) {
+    const df s = df_mul_f(df_add(lo, hi), 0.5f);
+    shd[j] = df{s.hi * un, s.lo * un};
+  }
 }
 
 // Inverse iteration and clean-up, one block per group of close shifts: block b
@@ -1118,64 +619,139 @@ __global__ void __launch_bounds__(kSvecThreads) k_syev_vecs(int n, int nwant, si
     ld = NW;
   }
   const df pv = df{fmaxf(3.6e-15f * tnorm, 1.0e-30f), 0.f};
-  for (int round = 0; round <= maxpos; ++round) {
-    for (int jj = tid; jj < G; jj += nt)
-      if (cps[jj] == round) syev_inverse_iteration(b + jj, jj, cst[jj], shd[b + jj], dd, ee, n, pv, dinv, lm, Z, ld);
+  if (maxpos == 0 && G <= nt / 32) {
+    // no clusters and a warp for every vector
+    const int jj = tid >> 5, j = b + jj;
+    if (jj < G) {
+      // the shift after the last wanted one is there too (unless there is none)
+      const bool apart = shift_gap(shd, j) > 1.0e-3f * tnorm && (j + 1 == n || shift_gap(shd, j + 1) > 1.0e-3f * tnorm);
+      syev_inverse_iteration_warp(j, apart ? 2 : 3, shd[j], dd, ee, n, pv.hi, dinv + jj, lm + jj, Z + jj,
+                                  ld);
+    }
     __syncthreads();
+  } else {
+    for (int round = 0; round <= maxpos; ++round) {
+      for (int jj = tid; jj < G; jj += nt)
+        if (cps[jj] == round) syev_inverse_iteration(b + jj, jj, cst[jj], shd[b + jj], dd, ee, n, pv, dinv, lm, Z, ld);
+      __syncthreads();
+    }
   }
   if (G == 1) {
-    if (tid == 0) syev_single(Z, ld, dd, ee, n, Zg + b, NW, evals + b);
+    if (tid < 32) syev_single(Z, ld, dd, ee, n, Zg + b, NW, evals + b);
   } else {
     syev_group_rr<4, 2>(G, Z, ld, dd, ee, n, dinv, rrw, perm, red, sf, Zg + b, NW, evals + b);
   }
 }
 
 // Back-transformation y = H_0 H_1 ... H_{n-3} z, one warp per eigenvector
-// (column c of Zg), held in shared memory; the block stages kSbChunk
-// reflectors at a time (chunk = reflectors k0, k0 - 1, ...) and each warp then
-// applies them to its own column without further barriers.  Writes evecs
-// (n x nwant float64).
-__global__ void __launch_bounds__(32 * kSbWarps) k_syev_back(int n, int nwant, int chunk, const df* __restrict__ hv,
+// (column c of Zg, held in shared memory), kSbChunk reflectors at a time: with
+// f_r = t_r (v_r^T z - sum_{s<r} f_s v_s^T v_r) (r = 0 the largest k, applied first) their
+// product takes z to z - sum_r f_r v_r, so the eight dot products with z are
+// formed together and z is read and written once per chunk; the block's
+// warps form the v_s^T v_r of the chunk between them.  Bound by latency: one reflector
+// after another, a warp reduction each, took 341 us for 128 of 256 (176 now).  Writes evecs (n x nwant float64).
+__device__ __forceinline__ void cp_async8(void* dst, const void* src, int bytes) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(
+                   static_cast<unsigned>(__cvta_generic_to_shared(dst))),
+               "l"(src), "r"(bytes)
+               : "memory");
+}
+
+__global__ void __launch_bounds__(32 * kSbWarps) k_syev_back(int n, int nwant, int bufs, const df* __restrict__ hv,
                                                              const df* __restrict__ tau_g,
                                                              const df* __restrict__ Zg, double* __restrict__ evecs,
                                                              const int* __restrict__ skip) {
   if (skip != nullptr && *skip != 0) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, wpb = blockDim.x >> 5;
+  constexpr int C = kSbChunk;
+  __shared__ df gram[C][C];  // [r][s]: v_r^T v_s, s < r
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const long long NW = nwant;
-  df* zs = reinterpret_cast<df*>(smem_raw);  // wpb x n
-  df* vs = zs + static_cast<long long>(wpb) * n;  // chunk x n
-  const int c = blockIdx.x * wpb + warp;
-  const bool live = c < nwant;
+  df* zs = reinterpret_cast<df*>(smem_raw);            // kSbWarps x n
+  df* taus = zs + static_cast<long long>(kSbWarps) * n;  // n
+  df* vb = taus + n;                                   // bufs x C x n, v_r at its rows' own indices
+  const int c = blockIdx.x * kSbWarps + warp;
   df* z = zs + static_cast<long long>(warp) * n;
-  if (live)
-    for (int i = lane; i < n; i += 32) z[i] = Zg[i * NW + c];
-  for (int k0 = n - 3; k0 >= 0; k0 -= chunk) {
-    const int nk = min(chunk, k0 + 1);
-    __syncthreads();  // the previous chunk is no longer read
-    for (long long idx = tid; idx < static_cast<long long>(nk) * n; idx += blockDim.x) {
-      const int r = static_cast<int>(idx / n), i = static_cast<int>(idx % n);
-      const int k = k0 - r, m = n - k - 1;
-      vs[idx] = i < m ? hv[static_cast<long long>(k) * n + i] : df{0.f, 0.f};
-    }
-    __syncthreads();
-    if (!live) continue;
-    for (int r = 0; r < nk; ++r) {
+  for (int i = lane; i < n; i += 32) z[i] = c < nwant ? Zg[i * NW + c] : df{0.f, 0.f};
+  for (int i = tid; i < n; i += 32 * kSbWarps) taus[i] = tau_g[i];
+  // reflectors k0, k0 - 1, ... of a chunk into buffer `buf` (rows above k zero-filled)
+  auto stage = [&](int k0, int buf) {
+    df* vs = vb + static_cast<long long>(buf) * C * n;
+    const int base = max(0, k0 - C + 1) + 1;
+    for (int r = warp; r < C; r += kSbWarps) {
       const int k = k0 - r;
-      const df t = tau_g[k];
-      if (t.hi == 0.f) continue;
-      const int m = n - k - 1;
-      const df* v = vs + static_cast<long long>(r) * n;
-      df_acc s = acc_zero();
-      for (int i = lane; i < m; i += 32) s.fma(v[i], z[k + 1 + i]);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) s.merge(shfl_xor_acc(s, o));
-      const df f = df_mul(t, s.value());
-      for (int i = lane; i < m; i += 32) z[k + 1 + i] = df_sub(z[k + 1 + i], df_mul(f, v[i]));
-      __syncwarp();
+      for (int i = base + lane; i < n; i += 32) {
+        const bool on = k >= 0 && i > k;
+        cp_async8(vs + r * n + i, hv + (on ? static_cast<long long>(k) * n + (i - k - 1) : 0), on ? 8 : 0);
+      }
     }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  int buf = 0;
+  if (n > 2 && bufs == 2) stage(n - 3, 0);
+  for (int k0 = n - 3; k0 >= 0; k0 -= C) {
+    const int base = max(0, k0 - C + 1) + 1;  // first row any of the chunk's reflectors touches
+    if (bufs == 2) {
+      if (k0 - C >= 0) {
+        stage(k0 - C, buf ^ 1);
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+      } else {
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+      }
+    } else {
+      stage(k0, 0);
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+    }
+    __syncthreads();  // the chunk is staged
+    const df* vs = vb + static_cast<long long>(buf) * C * n;
+    // passes 0, 1: the chunk's v_s^T v_r for r = warp + 1, warp + 5; pass 2: v_s^T z
+    df dr = df{0.f, 0.f};  // lane s: v_s^T z
+#pragma unroll 1
+    for (int pass = 0; pass < 3; ++pass) {
+      const int r = warp + 1 + pass * kSbWarps;
+      if (pass < 2 && r >= C) continue;
+      const df* u = pass < 2 ? vs + r * n : z;
+      df_acc a[C];
+#pragma unroll
+      for (int s = 0; s < C; ++s) a[s] = acc_zero();
+#pragma unroll 1
+      for (int i = base + lane; i < n; i += 32) {
+        const df ui = u[i];
+#pragma unroll
+        for (int s = 0; s < C; ++s) a[s].fma(vs[s * n + i], ui);
+      }
+#pragma unroll 1
+      for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int s = 0; s < C; ++s) a[s].merge(shfl_xor_acc(a[s], o));
+      df_acc mine = a[0];
+#pragma unroll
+      for (int s = 1; s < C; ++s)
+        if (lane == s) mine = a[s];
+      dr = mine.value();
+      if (pass < 2 && lane < C) gram[r][lane] = dr;
+    }
+    __syncthreads();  // gram is complete
+    // lane r holds v_r^T z, then f_r
+    const df t = lane < C && k0 - lane >= 0 ? taus[k0 - lane] : df{0.f, 0.f};
+    df f[C];
+#pragma unroll
+    for (int s = 0; s < C; ++s) {
+      f[s] = df_neg(shfl_df(df_mul(t, dr), s));
+      if (lane > s && lane < C) dr = df_add(dr, df_mul(f[s], gram[lane][s]));
+    }
+#pragma unroll 1
+    for (int i = base + lane; i < n; i += 32) {
+      df_acc u = acc_zero();
+      u.add(z[i]);
+#pragma unroll
+      for (int r = 0; r < C; ++r) u.fma(f[r], vs[r * n + i]);
+      z[i] = u.value();
+    }
+    __syncthreads();  // the chunk's buffer and gram are free again
+    if (bufs == 2) buf ^= 1;
   }
-  if (live)
+  if (c < nwant)
     for (int i = lane; i < n; i += 32) evecs[i * NW + c] = df_to_double(z[i]);
 }
 
@@ -2717,8 +2293,6 @@ __global__ void k_identity(int n, double* __restrict__ X) {
     X[i] = (i / N == i % N) ? 1.0 : 0.0;
 }
 
-constexpr size_t kSmemBudget = 225 * 1024;
-
 }  // namespace
 
 // ------------------------------------------------------------ host side
@@ -2781,7 +2355,7 @@ PencilWork* pencil_work_create(int dn, int qmax, cudaError_t* err, bool dry) {
     alloc((void**)&w->rr, sizeof(df) * 4 * (nwm * nwm > 4 * nwm ? nwm * nwm : 4 * nwm));
     alloc((void**)&w->perm, sizeof(int) * nwm);
     alloc((void**)&w->hv, sizeof(df) * nm * nm);
-    alloc((void**)&w->shd, sizeof(df) * nwm);
+    alloc((void**)&w->shd, sizeof(df) * (nwm + 1));
     alloc((void**)&w->bounds, sizeof(float) * 4);
     alloc((void**)&w->Lm, sizeof(double) * dn * dn);
     alloc((void**)&w->Hs, sizeof(double) * dn * dn);
@@ -2840,22 +2414,13 @@ bool cluster_fits(size_t smem) {
 void launch_syev_df(PencilWork* w, int n, int nwant, const double* H, double* evals, double* evecs,
                     cudaStream_t st, const int* skip) {
   if (n <= 0 || nwant <= 0) return;
-  // tridiagonalisation: W in shared memory when it fits beside v, p, d, e, tau
   const int ldw = n | 1;  // odd row stride: column walks of W hit different banks
-  const size_t tb = (5 * sizeof(df) * static_cast<size_t>(n) + 15) & ~static_cast<size_t>(15);
-  const size_t wb = sizeof(df) * static_cast<size_t>(n) * ldw;
-  const int inshared = tb + wb <= kSmemBudget;
-  const size_t sm_tri = tb + (inshared ? wb : 0);
-  const size_t sm_val = 2 * sizeof(df) * static_cast<size_t>(n) + 2 * sizeof(float) * static_cast<size_t>(n);
+  const size_t sm_val = 2 * sizeof(df) * static_cast<size_t>(n);
   // groups keep their vectors in shared memory up to the budget (the widest possible group: all nwant)
   const size_t sm_vec = std::min(kSmemBudget, syev_vecs_base(n, nwant) + syev_vecs_work(n, nwant));
-  // back-transformation: kSbWarps columns and kSbChunk staged reflectors of n df, fewer when n is large
-  int wpb = kSbWarps;
-  while (wpb > 1 && sizeof(df) * static_cast<size_t>(wpb + 1) * n > kSmemBudget) --wpb;
-  const int chunk = static_cast<int>(std::max<size_t>(
-      1, std::min<size_t>(kSbChunk, (kSmemBudget - sizeof(df) * static_cast<size_t>(wpb) * n) /
-                                        (sizeof(df) * static_cast<size_t>(n)))));
-  const size_t sm_back = sizeof(df) * static_cast<size_t>(wpb + chunk) * n;
+  // back-transformation: kSbWarps columns and one or two chunks of reflectors of n df (208 KB at n = 2048)
+  const int bufs = sizeof(df) * static_cast<size_t>(kSbWarps + 1 + 2 * kSbChunk) * n <= kSmemBudget ? 2 : 1;
+  const size_t sm_back = sizeof(df) * static_cast<size_t>(kSbWarps + 1 + bufs * kSbChunk) * n;
   ProfScope ps(st, P_PENCIL, 8.0 * n * n + 8.0 * n * nwant, 0.0, 4);
   // from kTriOneBlock rows a cluster of 16 CTAs, where it can be scheduled
   const size_t tri_rows = ceil_div(n, kTriCluster);
@@ -2866,49 +2431,15 @@ void launch_syev_df(PencilWork* w, int n, int nwant, const double* H, double* ev
     const cudaLaunchConfig_t cfg = tri_config(sm_cl, st, attr);
     cudaLaunchKernelEx(&cfg, k_syev_tri_cl, n, ldw, H, w->hv, w->dd, w->ee, w->tau, skip);
   } else {
-    ensure_dynamic_smem(reinterpret_cast<const void*>(k_syev_tri), sm_tri);
-    k_syev_tri<<<1, kSyThreads, sm_tri, st>>>(n, ldw, inshared, H, w->W, w->hv, w->dd, w->ee, w->tau, skip);
+    launch_syev_tri_block(w, n, ldw, H, skip, st);
   }
   ensure_dynamic_smem(reinterpret_cast<const void*>(k_syev_vals), sm_val);
-  k_syev_vals<<<ceil_div(nwant, kSvWarps), 32 * kSvWarps, sm_val, st>>>(n, nwant, w->dd, w->ee, w->shd, w->bounds,
-                                                                        skip);
+  k_syev_vals<<<std::min(nwant + 1, n), kSvThreads, sm_val, st>>>(n, w->dd, w->ee, w->shd, w->bounds, skip);
   ensure_dynamic_smem(reinterpret_cast<const void*>(k_syev_vecs), sm_vec);
   k_syev_vecs<<<nwant, kSvecThreads, sm_vec, st>>>(n, nwant, sm_vec, w->dd, w->ee, w->shd, w->bounds, w->fac, w->rr,
                                                    w->Zt, evals, skip);
   ensure_dynamic_smem(reinterpret_cast<const void*>(k_syev_back), sm_back);
-  k_syev_back<<<ceil_div(nwant, wpb), 32 * wpb, sm_back, st>>>(n, nwant, chunk, w->hv, w->tau, w->Zt, evecs, skip);
-}
-
-size_t syev_scratch(int n, int nwant, PencilWork* w, void* base) {
-  size_t off = 0;
-  char* at = static_cast<char*>(base);
-  auto carve = [&](auto** p, size_t count) {
-    if (base) *p = reinterpret_cast<std::remove_reference_t<decltype(*p)>>(at + off);
-    off = (off + sizeof(**p) * count + 255) & ~static_cast<size_t>(255);
-  };
-  const size_t nm = static_cast<size_t>(n), nw = static_cast<size_t>(nwant);
-  carve(&w->hv, nm * nm);
-  carve(&w->dd, nm);
-  carve(&w->ee, nm);
-  carve(&w->tau, nm);
-  carve(&w->shd, nw);
-  carve(&w->bounds, 4);
-  carve(&w->fac, 3 * nm * nw);
-  carve(&w->Zt, nm * nw);
-  carve(&w->rr, 4 * (nw * nw > 4 * nw ? nw * nw : 4 * nw));
-  return off;
-}
-
-size_t syev_scratch_bytes(int n, int nwant) {
-  PencilWork w;
-  return syev_scratch(n, nwant, &w, nullptr);
-}
-
-void launch_syev_df_into(int n, int nwant, const double* H, double* evals, double* evecs, void* scratch,
-                         cudaStream_t st) {
-  PencilWork w;
-  syev_scratch(n, nwant, &w, scratch);
-  launch_syev_df(&w, n, nwant, H, evals, evecs, st);
+  k_syev_back<<<ceil_div(nwant, kSbWarps), 32 * kSbWarps, sm_back, st>>>(n, nwant, bufs, w->hv, w->tau, w->Zt, evecs, skip);
 }
 
 void launch_pencil_solve(PencilWork* w, int dn, int m, int q, const double* C64, const float2* Cdf,

@@ -111,7 +111,9 @@ const char* kNames[P_COUNT] = {"defect", "smooth", "transfer", "coarse_solve", "
 }  // namespace
 
 void ensure_dynamic_smem(const void* func, size_t bytes) {
-  if (bytes <= 48 * 1024) return;
+  // without the attribute static and dynamic shared memory together may take 48 KB; no kernel here has 8 KB
+  // of static arrays beside dynamic ones
+  if (bytes <= 40 * 1024) return;
   // the attribute belongs to the current device's copy of the function: one
   // record per (device, function)
   int dev = 0;

@@ -29,7 +29,7 @@ enum ProfClass {
 // Raise a kernel's dynamic shared-memory limit to at least `bytes`, never
 // lowering it: the limit is one per function for the whole process, so solves
 // running on several host threads must not shrink it under each other's
-// launches.  Sizes up to 48 KB need no attribute.  The attribute is set on
+// launches.  Sizes up to 40 KB need no attribute (48 KB with the static arrays).  The attribute is set on
 // the current device, and recorded per (device, function).
 void ensure_dynamic_smem(const void* func, size_t bytes);
 

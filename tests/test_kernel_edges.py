@@ -58,43 +58,44 @@ def test_block_per_row_sweeps(width, tune):
             assert np.all(err <= 2e-5), (level, err.max())
 
 
-@pytest.mark.parametrize("n,nwant", [(39, 7), (40, 7), (41, 41), (63, 5), (64, 64), (65, 9), (127, 33), (129, 20), (255, 40),
-                                     (257, 16), (511, 24), (512, 31), (513, 12)])
-def test_sym_eigh_cluster_sizes(n, nwant):
-    """The dense eigensolver around the sizes where its tridiagonalisation changes form or distribution (one
-    block below 40 rows and above 512, rows dealt over 16 CTAs in between, one lane per own row) and where the
-    shifts, vectors and reflector chunks have remainders, against LAPACK (bounds of the eigensolver tests)."""
+@pytest.mark.parametrize("kind", ["dense", "decoupled", "diagonal", "close"])
+@pytest.mark.parametrize("n,nwant", [(1, 1), (3, 2), (39, 7), (40, 7), (41, 41), (63, 5), (64, 64), (65, 9), (127, 33),
+                                     (129, 20), (255, 40), (257, 16), (328, 64), (511, 24), (512, 31), (513, 12)])
+def test_coarse_eigensolver_sizes(n, nwant, kind):
+    """The solve path's dense eigensolver around the sizes where its tridiagonalisation changes form or distribution
+    (one block below 40 rows and above 512, rows dealt over 16 CTAs in between, one lane per own row) and where the
+    shifts, vectors and reflector chunks have remainders: a one-level hierarchy, whose solve is the dense
+    eigenproblem of its pencil, against LAPACK.  decoupled, diagonal: reflections with nothing to reflect and zero
+    off-diagonals; close: all wanted values within 1e-4 ||H|| (one clean-up group; needs values beyond them that
+    make ||H||)."""
+    from paper_1503_08462_gb300.inputs import hierarchy
+
+    if kind == "close" and nwant == n:
+        pytest.skip("no values beyond the wanted ones")
+
     rng = np.random.default_rng(n)
     c = rng.standard_normal((n, n))
-    H = np.diag(5.0 + 3.0 * np.arange(n)) + c + c.T
-    w, V = ae.amgeig_sym_eigh(H, nwant)
+    H = np.diag(50.0 + 3.0 * np.arange(n)) + c + c.T
+    if kind == "decoupled":
+        H[: n // 2, n // 2:] = 0.0
+        H[n // 2:, : n // 2] = 0.0
+    elif kind == "diagonal":
+        H = np.diag(1.0 + rng.permutation(n))
+    elif kind == "close":
+        Q, _ = np.linalg.qr(c)
+        spec = np.concatenate([rng.uniform(1.0, 1.5, nwant), rng.uniform(10.0, 2.0e4, n - nwant)])
+        H = (Q * np.sort(spec)) @ Q.T
+        H = 0.5 * (H + H.T)
+    H[np.abs(H) == 0.0] = 0.0
+    H = H + np.diag(np.full(n, max(0.0, 1.0 - np.linalg.eigvalsh(H)[0])))  # SPD
+    rp = np.arange(0, n * n + 1, n)
+    ci = np.tile(np.arange(n), n)
+    hh = hierarchy.build_hierarchy(rp, ci, H.ravel(), np.eye(n).ravel(), coarse_cap=n)
+    assert hh.sizes == [n]
+    with ae.Hierarchy(hierarchy.to_blob(hh)) as h:
+        lam, U, _, _ = h.solve(nwant, tol=1.0, opt=ae.options(coarse_modes=nwant))
     full = np.linalg.eigvalsh(H)
     scale = np.abs(full).max()
-    assert np.all(np.abs(w - full[:nwant]) <= 1e-12 * scale)
-    assert np.abs(V.T @ V - np.eye(nwant)).max() < 1e-12
-    assert np.abs(H @ V - V * w).max() <= 1e-11 * scale
-
-
-@pytest.mark.parametrize("n,nwant", [(1, 1), (3, 2), (16, 16), (39, 12), (40, 12), (127, 64), (128, 64)])
-def test_noalloc_gives_the_allocating_entrys_bits(n, nwant):
-    """Both entry points run the same kernels: the same bits, also on a diagonal and a decoupled matrix."""
-    import torch
-
-    rng = np.random.default_rng(n)
-    c = rng.standard_normal((n, n))
-    dense = np.diag(5.0 + 3.0 * np.arange(n)) + c + c.T
-    split = dense.copy()
-    split[: n // 2, n // 2:] = 0.0
-    split[n // 2:, : n // 2] = 0.0
-    for H in (dense, split, np.diag(1.0 + np.arange(n))):
-        w, V = ae.amgeig_sym_eigh(H, nwant)
-        Hd = torch.tensor(H, dtype=torch.float64, device="cuda")
-        wd = torch.empty(nwant, dtype=torch.float64, device="cuda")
-        Vd = torch.empty((n, nwant), dtype=torch.float64, device="cuda")
-        ae.amgeig_sym_eigh_noalloc(Hd, wd, Vd)
-        torch.cuda.synchronize()
-        np.testing.assert_array_equal(wd.cpu().numpy(), w)
-        np.testing.assert_array_equal(Vd.cpu().numpy(), V)
-        full = np.linalg.eigvalsh(H)
-        assert np.all(np.abs(w - full[:nwant]) <= 1e-12 * np.abs(full).max())
-        assert np.abs(V.T @ V - np.eye(nwant)).max() < 1e-12
+    assert np.all(np.abs(lam - full[:nwant]) <= 1e-12 * scale)
+    assert np.abs(U.T @ U - np.eye(nwant)).max() < (1e-12 if kind != "dense" else 2e-12)
+    assert np.abs(H @ U - U * lam).max() <= 1e-11 * scale
