@@ -22,7 +22,7 @@
 //   the same Rayleigh-Ritz problem (same eigenvalues as the paper's pencil),
 //   only better conditioned, and everything runs in float-float.
 // * The symmetric eigenproblem is solved in float-float (48-bit significand):
-//   Householder tridiagonalisation (one 1024-thread block), bisection with
+//   Householder tridiagonalisation (a thread-block cluster), bisection with
 //   Sturm counts for the wanted eigenvalues (float32), each shift refined by
 //   float-float Sturm multisection, inverse iteration in float-float
 //   (Gram-Schmidt inside clusters of nearly equal shifts), a Rayleigh-Ritz
