@@ -227,8 +227,8 @@ __device__ void syev_single(const df* Z, long long ldz, const df* dd, const df* 
 // eigenvectors Zg (n x nwant df).
 constexpr int kSvThreads = 128;  // points per round of k_syev_vals
 constexpr int kSvecThreads = 512;
-constexpr int kSbWarps = 4;  // eigenvectors per block of k_syev_back
-constexpr int kSbChunk = 8;  // reflectors applied together in k_syev_back
+constexpr int kSbWarps = 4;  // eigenvectors per block of k_syev_back (one where four do not fit)
+constexpr int kSbChunk = 8;  // reflectors applied together in k_syev_back (four where eight do not fit)
 
 // Householder tridiagonalisation by a thread-block cluster of 16 CTAs, row i of W in CTA
 // i % 16's shared memory (dealt cyclically, so the shrinking trailing block stays
@@ -644,12 +644,14 @@ __global__ void __launch_bounds__(kSvecThreads) k_syev_vecs(int n, int nwant, si
 }
 
 // Back-transformation y = H_0 H_1 ... H_{n-3} z, one warp per eigenvector
-// (column c of Zg, held in shared memory), kSbChunk reflectors at a time: with
+// (column c of Zg, held in shared memory), C reflectors at a time: with
 // f_r = t_r (v_r^T z - sum_{s<r} f_s v_s^T v_r) (r = 0 the largest k, applied first) their
-// product takes z to z - sum_r f_r v_r, so the eight dot products with z are
+// product takes z to z - sum_r f_r v_r, so the C dot products with z are
 // formed together and z is read and written once per chunk; the block's
 // warps form the v_s^T v_r of the chunk between them.  Bound by latency: one reflector
-// after another, a warp reduction each, took 341 us for 128 of 256 (176 now).  Writes evecs (n x nwant float64).
+// after another, a warp reduction each, took 341 us for 128 of 256 (176 now).  WPB columns per block; the
+// columns, the reflectors' scalars and one or two chunks share a CTA's memory, so C and WPB
+// shrink with n (launch_syev_back).  Writes evecs (n x nwant float64).
 __device__ __forceinline__ void cp_async8(void* dst, const void* src, int bytes) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(
                    static_cast<unsigned>(__cvta_generic_to_shared(dst))),
@@ -657,28 +659,27 @@ __device__ __forceinline__ void cp_async8(void* dst, const void* src, int bytes)
                : "memory");
 }
 
-__global__ void __launch_bounds__(32 * kSbWarps) k_syev_back(int n, int nwant, int bufs, const df* __restrict__ hv,
-                                                             const df* __restrict__ tau_g,
-                                                             const df* __restrict__ Zg, double* __restrict__ evecs,
-                                                             const int* __restrict__ skip) {
+template <int C, int WPB>
+__global__ void __launch_bounds__(32 * WPB) k_syev_back(int n, int nwant, int bufs, const df* __restrict__ hv,
+                                                        const df* __restrict__ tau_g, const df* __restrict__ Zg,
+                                                        double* __restrict__ evecs, const int* __restrict__ skip) {
   if (skip != nullptr && *skip != 0) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  constexpr int C = kSbChunk;
   __shared__ df gram[C][C];  // [r][s]: v_r^T v_s, s < r
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const long long NW = nwant;
-  df* zs = reinterpret_cast<df*>(smem_raw);            // kSbWarps x n
-  df* taus = zs + static_cast<long long>(kSbWarps) * n;  // n
+  df* zs = reinterpret_cast<df*>(smem_raw);            // WPB x n
+  df* taus = zs + static_cast<long long>(WPB) * n;     // n
   df* vb = taus + n;                                   // bufs x C x n, v_r at its rows' own indices
-  const int c = blockIdx.x * kSbWarps + warp;
+  const int c = blockIdx.x * WPB + warp;
   df* z = zs + static_cast<long long>(warp) * n;
   for (int i = lane; i < n; i += 32) z[i] = c < nwant ? Zg[i * NW + c] : df{0.f, 0.f};
-  for (int i = tid; i < n; i += 32 * kSbWarps) taus[i] = tau_g[i];
+  for (int i = tid; i < n; i += 32 * WPB) taus[i] = tau_g[i];
   // reflectors k0, k0 - 1, ... of a chunk into buffer `buf` (rows above k zero-filled)
   auto stage = [&](int k0, int buf) {
     df* vs = vb + static_cast<long long>(buf) * C * n;
     const int base = max(0, k0 - C + 1) + 1;
-    for (int r = warp; r < C; r += kSbWarps) {
+    for (int r = warp; r < C; r += WPB) {
       const int k = k0 - r;
       for (int i = base + lane; i < n; i += 32) {
         const bool on = k >= 0 && i > k;
@@ -704,13 +705,14 @@ __global__ void __launch_bounds__(32 * kSbWarps) k_syev_back(int n, int nwant, i
     }
     __syncthreads();  // the chunk is staged
     const df* vs = vb + static_cast<long long>(buf) * C * n;
-    // passes 0, 1: the chunk's v_s^T v_r for r = warp + 1, warp + 5; pass 2: v_s^T z
+    // the passes before the last: the chunk's v_s^T v_r for r = warp + 1, warp + 1 + WPB, ...; the last: v_s^T z
+    constexpr int kLast = (C - 1 + WPB - 1) / WPB;
     df dr = df{0.f, 0.f};  // lane s: v_s^T z
 #pragma unroll 1
-    for (int pass = 0; pass < 3; ++pass) {
-      const int r = warp + 1 + pass * kSbWarps;
-      if (pass < 2 && r >= C) continue;
-      const df* u = pass < 2 ? vs + r * n : z;
+    for (int pass = 0; pass <= kLast; ++pass) {
+      const int r = warp + 1 + pass * WPB;
+      if (pass < kLast && r >= C) continue;
+      const df* u = pass < kLast ? vs + r * n : z;
       df_acc a[C];
 #pragma unroll
       for (int s = 0; s < C; ++s) a[s] = acc_zero();
@@ -729,7 +731,7 @@ __global__ void __launch_bounds__(32 * kSbWarps) k_syev_back(int n, int nwant, i
       for (int s = 1; s < C; ++s)
         if (lane == s) mine = a[s];
       dr = mine.value();
-      if (pass < 2 && lane < C) gram[r][lane] = dr;
+      if (pass < kLast && lane < C) gram[r][lane] = dr;
     }
     __syncthreads();  // gram is complete
     // lane r holds v_r^T z, then f_r
@@ -2411,6 +2413,31 @@ bool cluster_fits(size_t smem) {
   return ok;
 }
 
+// Shared memory of k_syev_back: WPB columns, the scalars, `bufs` chunks of C reflectors.
+size_t syev_back_smem(int n, int c, int wpb, int bufs) {
+  return sizeof(df) * static_cast<size_t>(wpb + 1 + bufs * c) * n;
+}
+
+template <int C, int WPB>
+void launch_syev_back_as(PencilWork* w, int n, int nwant, int bufs, double* evecs, cudaStream_t st, const int* skip) {
+  const size_t sm = syev_back_smem(n, C, WPB, bufs);
+  ensure_dynamic_smem(reinterpret_cast<const void*>(k_syev_back<C, WPB>), sm);
+  k_syev_back<C, WPB><<<ceil_div(nwant, WPB), 32 * WPB, sm, st>>>(n, nwant, bufs, w->hv, w->tau, w->Zt, evecs, skip);
+}
+
+// Eight reflectors and four columns per block while they fit (two chunks in flight up to 1371 rows, one up to
+// 2215), then four reflectors, and last one column per block: the largest coarsest level (4096
+// rows) with the widest border (128) takes 198 KB.
+void launch_syev_back(PencilWork* w, int n, int nwant, double* evecs, cudaStream_t st, const int* skip) {
+  const auto fits = [n](int c, int wpb, int bufs) { return syev_back_smem(n, c, wpb, bufs) <= kSmemBudget; };
+  if (fits(kSbChunk, kSbWarps, 1))
+    launch_syev_back_as<kSbChunk, kSbWarps>(w, n, nwant, fits(kSbChunk, kSbWarps, 2) ? 2 : 1, evecs, st, skip);
+  else if (fits(kSbChunk / 2, kSbWarps, 1))
+    launch_syev_back_as<kSbChunk / 2, kSbWarps>(w, n, nwant, 1, evecs, st, skip);
+  else
+    launch_syev_back_as<kSbChunk / 2, 1>(w, n, nwant, 1, evecs, st, skip);
+}
+
 void launch_syev_df(PencilWork* w, int n, int nwant, const double* H, double* evals, double* evecs,
                     cudaStream_t st, const int* skip) {
   if (n <= 0 || nwant <= 0) return;
@@ -2418,9 +2445,6 @@ void launch_syev_df(PencilWork* w, int n, int nwant, const double* H, double* ev
   const size_t sm_val = 2 * sizeof(df) * static_cast<size_t>(n);
   // groups keep their vectors in shared memory up to the budget (the widest possible group: all nwant)
   const size_t sm_vec = std::min(kSmemBudget, syev_vecs_base(n, nwant) + syev_vecs_work(n, nwant));
-  // back-transformation: kSbWarps columns and one or two chunks of reflectors of n df (208 KB at n = 2048)
-  const int bufs = sizeof(df) * static_cast<size_t>(kSbWarps + 1 + 2 * kSbChunk) * n <= kSmemBudget ? 2 : 1;
-  const size_t sm_back = sizeof(df) * static_cast<size_t>(kSbWarps + 1 + bufs * kSbChunk) * n;
   ProfScope ps(st, P_PENCIL, 8.0 * n * n + 8.0 * n * nwant, 0.0, 4);
   // from kTriOneBlock rows a cluster of 16 CTAs, where it can be scheduled
   const size_t tri_rows = ceil_div(n, kTriCluster);
@@ -2438,8 +2462,7 @@ void launch_syev_df(PencilWork* w, int n, int nwant, const double* H, double* ev
   ensure_dynamic_smem(reinterpret_cast<const void*>(k_syev_vecs), sm_vec);
   k_syev_vecs<<<nwant, kSvecThreads, sm_vec, st>>>(n, nwant, sm_vec, w->dd, w->ee, w->shd, w->bounds, w->fac, w->rr,
                                                    w->Zt, evals, skip);
-  ensure_dynamic_smem(reinterpret_cast<const void*>(k_syev_back), sm_back);
-  k_syev_back<<<ceil_div(nwant, kSbWarps), 32 * kSbWarps, sm_back, st>>>(n, nwant, bufs, w->hv, w->tau, w->Zt, evecs, skip);
+  launch_syev_back(w, n, nwant, evecs, st, skip);
 }
 
 void launch_pencil_solve(PencilWork* w, int dn, int m, int q, const double* C64, const float2* Cdf,

@@ -99,3 +99,51 @@ def test_coarse_eigensolver_sizes(n, nwant, kind):
     assert np.all(np.abs(lam - full[:nwant]) <= 1e-12 * scale)
     assert np.abs(U.T @ U - np.eye(nwant)).max() < (1e-12 if kind != "dense" else 2e-12)
     assert np.abs(H @ U - U * lam).max() <= 1e-11 * scale
+
+
+def _one_level(rp, ci, vals, n):
+    """A one-level hierarchy of the pencil (A, I): its solve is the dense eigenproblem of A."""
+    from paper_1503_08462_gb300.inputs import hierarchy
+
+    mass = np.where(np.repeat(np.arange(n), np.diff(rp)) == ci, 1.0, 0.0)
+    hh = hierarchy.build_hierarchy(rp, ci, vals, mass, coarse_cap=n)
+    assert hh.sizes == [n]
+    return ae.Hierarchy(hierarchy.to_blob(hh))
+
+
+@pytest.mark.parametrize("a,b,nwant", [(43, 51, 6), (45, 50, 6), (50, 64, 5), (53, 61, 5)])
+def test_coarse_eigensolver_large_levels(a, b, nwant):
+    """One-level hierarchies of 2193, 2250, 3200 and 3233 rows: the back-transformation's columns and reflectors no
+    longer fit a CTA's shared memory eight and four at a time beyond 2215 rows, nor four and four beyond 3200.  The
+    a x b Dirichlet Laplacian has the eigenvalues 4 sin^2(pi i / (2a + 2)) + 4 sin^2(pi j / (2b + 2))."""
+    import scipy.sparse as sp
+
+    def line(n):
+        return sp.diags([-np.ones(n - 1), 2.0 * np.ones(n), -np.ones(n - 1)], [-1, 0, 1])
+
+    n = a * b
+    A = (sp.kron(line(a), sp.identity(b)) + sp.kron(sp.identity(a), line(b))).tocsr()
+    A.sort_indices()
+    with _one_level(A.indptr, A.indices, A.data, n) as h:
+        lam, U, _, _ = h.solve(nwant, tol=1.0, opt=ae.options(coarse_modes=nwant))
+    si, sj = (4.0 * np.sin(np.pi * np.arange(1, k + 1) / (2 * k + 2)) ** 2 for k in (a, b))
+    ref = np.sort((si[:, None] + sj[None, :]).ravel())[:nwant]
+    # as test_coarse_eigensolver_sizes, in units of ||A|| < 8; rounding of the n reflections grows with sqrt(n)
+    assert np.all(np.abs(lam - ref) <= 1e-11)
+    assert np.abs(U.T @ U - np.eye(nwant)).max() < 1e-11
+    assert np.abs(A @ U - U * lam).max() <= 1e-10
+
+
+def test_dense_pencil_beyond_the_largest_chunk():
+    """A correction whose pencil (2144 coarse modes and 90 columns, 2234 rows) passes 2215 rows while its coarsest
+    level does not, against the oracle's iterate (float64 path)."""
+    p, blob, hh = problem_and_blob("square", 66, 2230, 1)
+    assert hh.sizes[-1] <= 2215 < hh.sizes[-1] + 90
+    oh = O.read_blob(blob)
+    q, kw = 80, dict(q_extra=10, fixed_corrections=1, coarse_modes=0)
+    lam_o, _, _ = O.solve(oh, q, tol=0.0, opts=O.Options(**kw))
+    with ae.Hierarchy(blob) as h:
+        lam, U, info, _ = h.solve(q, tol=0.0, opt=ae.options(**kw))
+    assert info.dense_fallbacks > 0
+    assert np.all(np.abs(lam - lam_o) / lam_o < eig_rel_tol(lam_o, lam_max(p)))
+    assert np.max(np.abs(U.T @ (oh.M[0] @ U) - np.eye(q))) < 1e-10
