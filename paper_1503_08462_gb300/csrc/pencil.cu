@@ -58,22 +58,27 @@ __device__ __forceinline__ df_acc warp_acc_sum(df_acc a) {
 // leading principal minors p_i = (d_i - x) p_{i-1} - e_{i-1}^2 p_{i-2} (Golub & Van Loan
 // 8.4.1): a sign change per eigenvalue.  The recurrence's chain is one product
 // and one difference (~75 cycles in float-float) where the quotient form
-// q_i = d_i - x - e^2 / q_{i-1} adds a reciprocal (~300).  The minors' range is kept by an
-// exact power-of-two rescaling of the pair every other step; d and e^2 are
-// scaled to ||T|| <= 1, so a step grows them by at most 3.  A zero minor is
-// replaced by a tiny one of the opposite sign (one count, as for a tiny negative pivot).
+// q_i = d_i - x - e^2 / q_{i-1} adds a reciprocal (~300).  d and e^2 are scaled to ||T|| <= 1, so
+// a step grows the minors by at most 3, and their range is kept by an exact power-of-two
+// rescaling of the pair every other step, to 2^100.  A minor below 2^-60 of the one before (a
+// pivot that small moves d_i by 2^-60 ||T||, far below the shifts' tolerance) becomes -2^-60 of it, a
+// tiny negative pivot: so a rescaled pair is at least (2^100, 2^40), the next two minors at least 2^-20 and
+// 2^-80, and no run of equal decoupled entries at x can take the minors to zero.
+constexpr float kMinorTop = 1.2676506e30f;     // 2^100
+constexpr float kMinorFloor = 8.6736174e-19f;  // 2^-60
+
 __device__ __forceinline__ float minor_scale(float a, float b) {
   const int e = (__float_as_int(fmaxf(fabsf(a), fabsf(b))) >> 23) & 0xff;
-  return __int_as_float((254 - e) << 23);  // 2^(127 - e)
+  return __int_as_float((354 - e) << 23);  // 2^(227 - e); the larger minor is at least 2^-20, so e >= 107
 }
 
 __device__ __forceinline__ int sturm_count(const df* d, const df* e2, int n, float x) {
-  float p0 = 1.f, p1 = d[0].hi - x;
-  if (p1 == 0.f) p1 = -8.7e-19f;
+  float p0 = kMinorTop, p1 = (d[0].hi - x) * kMinorTop;
+  if (fabsf(p1) < kMinorFloor * p0) p1 = -kMinorFloor * p0;
   int cnt = p1 < 0.f;
   for (int i = 1; i < n; ++i) {
     float pn = fmaf(d[i].hi - x, p1, -e2[i - 1].hi * p0);
-    if (pn == 0.f) pn = -8.7e-19f * p1;
+    if (fabsf(pn) < kMinorFloor * fabsf(p1)) pn = -kMinorFloor * p1;
     cnt += (pn < 0.f) != (p1 < 0.f);
     p0 = p1;
     p1 = pn;
@@ -93,13 +98,14 @@ __device__ __forceinline__ df df_sub_sloppy(df a, df b) {
 }
 
 __device__ __forceinline__ int sturm_count_df(const df* d, const df* e2, int n, df x) {
-  df p0 = df{1.f, 0.f}, p1 = df_sub(d[0], x);
-  if (p1.hi == 0.f) p1 = df{-8.7e-19f, 0.f};
+  const df t = df_sub(d[0], x);
+  df p0 = df{kMinorTop, 0.f}, p1 = df{t.hi * kMinorTop, t.lo * kMinorTop};
+  if (fabsf(p1.hi) < kMinorFloor * p0.hi) p1 = df{-kMinorFloor * p0.hi, 0.f};
   int cnt = p1.hi < 0.f;
 #pragma unroll 2
   for (int i = 1; i < n; ++i) {
     df pn = df_sub_sloppy(df_mul(df_sub(d[i], x), p1), df_mul(e2[i - 1], p0));
-    if (pn.hi == 0.f) pn = df{-8.7e-19f * p1.hi, 0.f};
+    if (fabsf(pn.hi) < kMinorFloor * fabsf(p1.hi)) pn = df{-kMinorFloor * p1.hi, 0.f};
     cnt += (pn.hi < 0.f) != (p1.hi < 0.f);
     p0 = p1;
     p1 = pn;

@@ -147,3 +147,34 @@ def test_dense_pencil_beyond_the_largest_chunk():
     assert info.dense_fallbacks > 0
     assert np.all(np.abs(lam - lam_o) / lam_o < eig_rel_tol(lam_o, lam_max(p)))
     assert np.max(np.abs(U.T @ (oh.M[0] @ U) - np.eye(q))) < 1e-10
+
+
+@pytest.mark.parametrize("lam,repeated", [(0.25, "0x1.00006daf5b7p-2"), (0.2718281828, "0x1.165a8baf5b7p-2"),
+                                          (0.3141592653, "0x1.41b365af5b7p-2")])
+def test_shift_beside_repeated_decoupled_values(lam, repeated):
+    """A diagonal matrix whose eight equal leading entries lie exactly on a counting point of the shift search for
+    the eigenvalue just below them (1.6e-6 ||H||, the spacing of the first float-float round) while its other
+    neighbour is outside its clean-up group: a count that stops at a run of vanishing minors loses the entries after
+    it, puts the shift on the repeated value and leaves the neighbour's vector in the result."""
+    n, nwant = 64, 16
+    d = 0.5 + 0.5 * (np.arange(n) + 1) / n
+    d[:8] = float.fromhex(repeated)
+    d[n - 9:n - 3] = 0.175 - 0.01 * np.arange(6)
+    d[n - 3], d[n - 2], d[n - 1] = lam - 2.4e-4, lam, 1.0
+    with _one_level(np.arange(n + 1), np.arange(n), d, n) as h:
+        w, U, _, _ = h.solve(nwant, tol=1.0, opt=ae.options(coarse_modes=nwant))
+    assert np.all(np.abs(w - np.sort(d)[:nwant]) <= 1e-12)
+    assert np.abs(U.T @ U - np.eye(nwant)).max() < 1e-12
+    assert np.abs(d[:, None] * U - U * w).max() <= 1e-11
+
+
+@pytest.mark.parametrize("n,nwant", [(5, 5), (24, 9), (65, 20), (200, 40), (512, 33)])
+@pytest.mark.parametrize("run", [2, 3])
+def test_coarse_eigensolver_repeated_values(n, nwant, run):
+    """Diagonal matrices whose values come in runs of 2 and 3: zero off-diagonals and groups of equal shifts."""
+    d = 1.0 - (np.arange(n) // run) / 512.0
+    with _one_level(np.arange(n + 1), np.arange(n), d, n) as h:
+        w, U, _, _ = h.solve(nwant, tol=1.0, opt=ae.options(coarse_modes=nwant))
+    assert np.all(np.abs(w - np.sort(d)[:nwant]) <= 1e-12)
+    assert np.abs(U.T @ U - np.eye(nwant)).max() < 1e-12
+    assert np.abs(d[:, None] * U - U * w).max() <= 1e-11
