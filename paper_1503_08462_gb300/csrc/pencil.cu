@@ -2047,11 +2047,17 @@ __global__ void __launch_bounds__(32 * kBackWarps) k_std_back(int m, int q, int 
 }
 
 // Xc = Z_m (a - B b) (d_n x p, also as float-float pairs in Xc2 when non-null) and Y = b (q x p) from
-// evecs = [a; b].  Each block takes kXcCols columns: it stages b, forms a - B b in shared memory and then
-// the d_n rows of the product, so that no work is repeated between blocks.
+// evecs = [a; b].  Block (x, y) takes kXcCols columns and the y-th of gridDim.y runs of rows: it stages b, forms
+// a - B b in shared memory and then its rows of the product.  Bound by the latency of the loads of B and Z_m,
+// so the rows are split over as many blocks as make 128 in all: a - B b is cheap to form again per run, and one block per
+// column pair for all rows left narrow borders on one to fourteen SMs.  Launch times on 287 coarse rows at
+// 1, 6, 14 and 28 columns, all rows in one run -> split: m = 64 15.5, 23.7, 24.8, 23.8 -> 9.6, 10.8, 12.7, 13.9 us;
+// m = 287 49.9, 85.4, 87, 83.5 -> 25.5, 32.4, 39.7, 44.1 us.
 // q: the border (columns of V), p: the pairs (columns of evecs, Xc and Y).
 constexpr int kXcCols = 2;
-constexpr int kXcThreads = 512;
+constexpr int kXcThreads = 256;
+constexpr int kXcBlocks = 128;  // blocks the rows are split for
+constexpr int kXcRows = 4;      // rows of a run at least
 
 __global__ void __launch_bounds__(kXcThreads) k_xc(int dn, int m, int q, int p, const float2* __restrict__ Zdf,
                                                    const df* __restrict__ KB, const double* __restrict__ evecs,
@@ -2059,6 +2065,7 @@ __global__ void __launch_bounds__(kXcThreads) k_xc(int dn, int m, int q, int p, 
                                                    double* __restrict__ Y) {
   extern __shared__ __align__(16) unsigned char xraw[];
   const int j0 = blockIdx.x * kXcCols, qc = min(kXcCols, p - j0);
+  const int rows = (dn + gridDim.y - 1) / gridDim.y, l0 = blockIdx.y * rows, l1 = min(dn, l0 + rows);
   df* bs = reinterpret_cast<df*>(xraw);  // q x kXcCols: b[:, j0:j0+qc]
   df* tmp = bs + q * kXcCols;            // m x kXcCols
   const int tid = threadIdx.x, nt = blockDim.x;
@@ -2067,7 +2074,7 @@ __global__ void __launch_bounds__(kXcThreads) k_xc(int dn, int m, int q, int p, 
     const int r = idx / qc, jj = idx % qc;
     const double v = evecs[static_cast<long long>(m + r) * p + j0 + jj];
     bs[r * kXcCols + jj] = to_df(v);
-    Y[r * p + j0 + jj] = v;
+    if (blockIdx.y == 0) Y[r * p + j0 + jj] = v;
   }
   __syncthreads();
   for (int idx = tid; idx < m * qc; idx += nt) {
@@ -2091,8 +2098,8 @@ __global__ void __launch_bounds__(kXcThreads) k_xc(int dn, int m, int q, int p, 
     tmp[i * kXcCols + jj] = df_sub(to_df(evecs[static_cast<long long>(i) * p + j0 + jj]), c0.value());
   }
   __syncthreads();
-  for (int idx = tid; idx < dn * qc; idx += nt) {
-    const int l = idx / qc, jj = idx % qc;
+  for (int idx = tid; idx < (l1 - l0) * qc; idx += nt) {
+    const int l = l0 + idx / qc, jj = idx % qc;
     const float2* zl = Zdf + static_cast<long long>(l) * dn;
     df_acc s0 = acc_zero(), s1 = acc_zero();
     int i = 0;
@@ -2532,7 +2539,9 @@ void launch_pencil_solve(PencilWork* w, int dn, int m, int q, const double* C64,
   k_std_back<<<ceil_div(p, kBackWarps), 32 * kBackWarps, bks, st>>>(m, q, p, w->Lq, w->Yh, skip);
   // Xc = Z_m (a - B b), Y = b
   smem_attr((const void*)k_xc, xsc);
-  k_xc<<<ceil_div(p, kXcCols), kXcThreads, xsc, st>>>(dn, m, q, p, Zdf, w->KB, w->Yh, Xc, Xcdf, Y);
+  const int cols = ceil_div(p, kXcCols);
+  const int runs = std::max(1, std::min(kXcBlocks / cols, ceil_div(dn, kXcRows)));
+  k_xc<<<dim3(cols, runs), kXcThreads, xsc, st>>>(dn, m, q, p, Zdf, w->KB, w->Yh, Xc, Xcdf, Y);
 }
 
 void launch_mass_factor(PencilWork* w, int dn, const double* Mn, int* status, cudaStream_t st) {

@@ -178,3 +178,19 @@ def test_coarse_eigensolver_repeated_values(n, nwant, run):
     assert np.all(np.abs(w - np.sort(d)[:nwant]) <= 1e-12)
     assert np.abs(U.T @ U - np.eye(nwant)).max() < 1e-12
     assert np.abs(d[:, None] * U - U * w).max() <= 1e-11
+
+
+@pytest.mark.parametrize("q,qe", [(1, 0), (2, 0), (1, 2), (6, 1), (11, 9), (20, 11)])
+@pytest.mark.parametrize("modes", [33, 0])
+def test_back_map_row_runs(q, qe, modes):
+    """Accepted corrections on an odd coarsest level whose rows the back-map splits into 37 to 8 runs for 1 to 31
+    columns, the last run short, against the oracle's iterates after one finest correction (float64 path; bounds of
+    the iteration parity tests)."""
+    p, blob, hh = problem_and_blob("square", 48, 300, 3)
+    oh = O.read_blob(blob)
+    kw = dict(q_extra=qe, fixed_corrections=1, coarse_modes=modes)
+    lam_o, _, _ = O.solve(oh, q, tol=0.0, opts=O.Options(**kw))
+    with ae.Hierarchy(blob) as h:
+        lam, U, _, _ = h.solve(q, tol=0.0, opt=ae.options(**kw))
+    assert np.all(np.abs(lam - lam_o) / lam_o < eig_rel_tol(lam_o, lam_max(p)))
+    assert np.max(np.abs(U.T @ (oh.M[0] @ U) - np.eye(q))) < 1e-10
