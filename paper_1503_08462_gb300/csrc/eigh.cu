@@ -928,6 +928,7 @@ static bool cluster_fits(int c, size_t bytes) {
   std::lock_guard<std::mutex> lk(mu);
   auto it = known.find({dev, key});
   if (it != known.end()) return it->second;
+  const cudaError_t before = cudaPeekAtLastError();
   ensure_dynamic_smem(reinterpret_cast<const void*>(k_syev_tri_cl), bytes);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(c);
@@ -942,7 +943,7 @@ static bool cluster_fits(int c, size_t bytes) {
   cfg.numAttrs = 1;
   int clusters = 0;
   const bool ok = cudaOccupancyMaxActiveClusters(&clusters, k_syev_tri_cl, &cfg) == cudaSuccess && clusters > 0;
-  if (!ok) cudaGetLastError();
+  if (!ok && before == cudaSuccess) cudaGetLastError();  // the answer is no; an earlier launch's error stays
   known[{dev, key}] = ok;
   return ok;
 }

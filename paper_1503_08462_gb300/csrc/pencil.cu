@@ -2414,6 +2414,7 @@ bool cluster_fits(size_t smem) {
   std::lock_guard<std::mutex> lk(mu);
   auto it = known.find(key);
   if (it != known.end()) return it->second;
+  const cudaError_t before = cudaPeekAtLastError();
   bool ok = cudaFuncSetAttribute(reinterpret_cast<const void*>(k_syev_tri_cl),
                                  cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
   ensure_dynamic_smem(reinterpret_cast<const void*>(k_syev_tri_cl), smem);
@@ -2421,7 +2422,7 @@ bool cluster_fits(size_t smem) {
   const cudaLaunchConfig_t cfg = tri_config(smem, nullptr, attr);
   int clusters = 0;
   ok = ok && cudaOccupancyMaxActiveClusters(&clusters, k_syev_tri_cl, &cfg) == cudaSuccess && clusters > 0;
-  if (!ok) cudaGetLastError();
+  if (!ok && before == cudaSuccess) cudaGetLastError();  // the answer is no; an earlier launch's error stays
   known[key] = ok;
   return ok;
 }
