@@ -1248,9 +1248,10 @@ TuneResult autotune_f4(DevCsr& S, int kind, int w4, const float* dinv, const flo
   }
   r.us = best;
   r.rule_us = time_us(rule);
-  if (by_row && cudaGetLastError() == cudaSuccess) {
+  const bool launched = cudaGetLastError() == cudaSuccess;  // asked once: a refused trial leaves the rule
+  if (launched && by_row) {
     S.tuned[w4] = 128;
-  } else if (r.G > 0 && cudaGetLastError() == cudaSuccess) {
+  } else if (launched && r.G > 0) {
     int lg = 0, ls = 0;
     while ((1 << lg) < r.G / r.S) ++lg;
     while ((1 << ls) < r.S) ++ls;

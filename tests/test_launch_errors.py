@@ -112,6 +112,14 @@ def run(tmp_path_factory):
     return call
 
 
+@pytest.mark.parametrize("w4", [1, 5, 8, 9, 16, 17, 20, 32])
+def test_refused_tuning_launch_leaves_the_rule(run, w4):
+    """A block-per-row trial whose launch is refused looks fastest (it takes no time); the operator must stay
+    untuned, as its shape does not fit the encoding of the others."""
+    assert run("tune-refused", w4) == 0
+    assert run("tune", w4) == 128  # the same trial, launched: chosen
+
+
 @pytest.mark.parametrize("solver", ["fits", "fits-entry"])
 def test_cluster_query_keeps_an_earlier_error(run, solver):
     """Asking whether a cluster can be resident (the answer is no, as an error) must not clear the error of an
