@@ -194,3 +194,58 @@ def test_back_map_row_runs(q, qe, modes):
         lam, U, _, _ = h.solve(q, tol=0.0, opt=ae.options(**kw))
     assert np.all(np.abs(lam - lam_o) / lam_o < eig_rel_tol(lam_o, lam_max(p)))
     assert np.max(np.abs(U.T @ (oh.M[0] @ U) - np.eye(q))) < 1e-10
+
+
+@pytest.mark.parametrize("width", [4, 20, 33, 128])
+def test_block_per_row_sweeps_bf16(width):
+    """The same sweeps on operators held in bfloat16, against the oracle's V-cycle on a hierarchy with the same
+    rounded values (bound of the bfloat16 V-cycle test)."""
+    import copy
+
+    import torch
+
+    def rounded(v):
+        return torch.from_numpy(v.astype(np.float32)).bfloat16().double().numpy()
+
+    _, blob, hh = problem_and_blob("cube", 20, 60, 4)
+    oh = O.read_blob(blob)
+    last = oh.n_levels - 1
+    assert any(oh.A[l].nnz >= 96 * oh.sizes[l] for l in range(last))
+    ob = copy.copy(oh)
+    ob.A, ob.P = [a.copy() for a in oh.A], [m.copy() for m in oh.P]
+    for l in range(last):
+        ob.A[l].data, ob.P[l].data = rounded(oh.A[l].data), rounded(oh.P[l].data)
+    ob.A[last] = oh.A[last]
+    ob.R = [m.T.tocsr() for m in ob.P]
+    ob.colour_cache = {}
+    rng = np.random.default_rng(width)
+    with ae.Hierarchy(blob) as h:
+        for level in range(last):
+            b = rng.standard_normal((oh.sizes[level], width))
+            ref = O.vcycle(ob, level, b, np.zeros_like(b))
+            x = ae.amgeig_apply_vcycle(h.handle, level, b, ae.options(precision=ae.AMGEIG_MIXED_BF16))
+            assert np.abs(x - ref).max() <= 2e-5 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("q,qe", [(1, 0), (10, 7), (20, 12)])
+def test_recombination_by_the_prolongation_chain(q, qe):
+    """The mixed path on a cube whose finest level (15,625 rows) recombines by the prolongation chain and whose next
+    (7,813 rows) by the composite, against the oracle's iterates after two finest corrections; bounds of the other
+    mixed iteration tests, the subspace up to its last gap of 1e-3."""
+    from helpers import m_subspace_angle
+
+    p, blob, _ = problem_and_blob("cube", 26, 400, 4)
+    oh = O.read_blob(blob)
+    composite = abs(oh.P[0])
+    for pl in oh.P[1:]:
+        composite = composite @ abs(pl)
+    assert oh.sizes[0] >= 8192 > oh.sizes[1] and composite.nnz > 4 * sum(pl.nnz for pl in oh.P)
+    kw = dict(q_extra=qe, fixed_corrections=2, v_cycles=2)
+    lam_o, U_o, _ = O.solve(oh, q, tol=0.0, opts=O.Options(**kw))
+    with ae.Hierarchy(blob) as h:
+        lam, U, _, _ = h.solve(q, tol=0.0, opt=ae.options(precision=ae.AMGEIG_MIXED_FP32, **kw))
+    gaps = np.append(np.diff(lam_o) / lam_o[1:], 1.0 if q == 1 else 0.0)
+    k = int(np.nonzero(gaps > 1e-3)[0].max()) + 1
+    assert np.max(np.abs(lam - lam_o) / lam_o) <= 1e-6
+    assert m_subspace_angle(U[:, :k], U_o[:, :k], oh.M[0]) <= 1e-4
+    assert np.abs(U.T @ (oh.M[0] @ U) - np.eye(q)).max() < 1e-10
