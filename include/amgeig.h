@@ -267,11 +267,12 @@ void amgeig_free_blob(void* blob);
 /* ---- building blocks, exposed for verification -------------------------- */
 
 /* The nwant smallest eigenpairs of the symmetric n x n matrix H (host, row-major,
- * float64), computed on device `device` by the solver's own dense eigensolver
- * (the black-box eigensolver of Algorithm 3.1 step 2: Householder
- * tridiagonalisation, Sturm bisection, inverse iteration and a Rayleigh-Ritz
- * clean-up, in float-float arithmetic).  evals: host, nwant doubles ascending;
- * evecs: host, n x nwant row-major, orthonormal columns.  1 <= nwant <= n <= 2048.
+ * float64), computed on device `device` (the method of the black-box
+ * eigensolver of Algorithm 3.1 step 2: Householder tridiagonalisation, Sturm
+ * bisection, inverse iteration and a Rayleigh-Ritz clean-up, in float-float
+ * arithmetic; solves run a faster form of it, kernels of their own).  evals:
+ * host, nwant doubles ascending; evecs: host, n x nwant row-major, orthonormal
+ * columns of unspecified sign.  1 <= nwant <= n <= 2048.
  * Errors: EINVAL, ENOMEM, ECUDA. */
 int amgeig_sym_eigh(int device, int n, int nwant, const double* H, double* evals, double* evecs);
 

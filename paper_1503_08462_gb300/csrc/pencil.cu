@@ -120,8 +120,8 @@ __device__ __forceinline__ int sturm_count_df(const df* d, const df* e2, int n, 
 
 // ------------------------------------------------------------ float-float syev
 //
-// Four kernels: the tridiagonalisation (k_syev_tri, one block, or k_syev_tri_cl,
-// a cluster of 16), the shifts (k_syev_vals), inverse iteration and clean-up
+// Four kernels: the tridiagonalisation (k_syev_tri_cl, a cluster of 16, or k_syev_tri of
+// eigh.cu, one block), the shifts (k_syev_vals), inverse iteration and clean-up
 // one block per group of close shifts (k_syev_vecs) and the
 // back-transformation (k_syev_back).
 

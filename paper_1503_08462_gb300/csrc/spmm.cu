@@ -294,7 +294,7 @@ struct F4Geo {
   // cpt = 0: one block of G = S * w4 threads per row (k_smooth_row), S streams of w4 lanes
 };
 
-// Streams of the block-per-row layout: blocks of 96-256 threads.
+// Streams of the block-per-row layout: blocks of 32 (one column lane) to 256 threads.
 int row_streams(int w4) { return w4 <= 8 ? 32 : w4 <= 16 ? 16 : 8; }
 // Whether a level's rows are long enough for it (see k_smooth_row)
 bool row_layout(long long rows, long long nnz) { return nnz >= 96 * rows && rows < 65536; }
